@@ -88,7 +88,7 @@ bool persistent_enabled() {
   return on;
 }
 
-// LBM_RESIDENT=0 keeps the on-chip resident steps out of the tuner's candidates.
+// LBM_RESIDENT=0 leaves the on-chip resident steps to explicit requests.
 bool resident_enabled() {
   static const bool on = [] {
     const char* e = std::getenv("LBM_RESIDENT");
@@ -309,6 +309,13 @@ lbm_status reserve_oc(Engine* E, const SetLayout& X) {
   return LBM_OK;
 }
 
+// The list's length, read after the stream has been synchronised.
+void take_seg_count(Engine* E) {
+  if (!E->nseg_copied) return;
+  E->nseg_copied = false;
+  E->seg_bound = *E->h_nseg;
+}
+
 lbm_status launch_pair(Engine* E, int moments) {
   // moments: 0 none, 1 into drho/ux/uy, 2 into drho/ux_prev/uy_prev
   const LatticeView* views = static_cast<const LatticeView*>(E->L.views.p);
@@ -402,26 +409,33 @@ lbm_status run_persistent(Engine* E, int64_t pairs) {
   return LBM_OK;
 }
 
-// One resident launch of n_steps steps (moments at the last step and, when
-// mom_prev >= 0, into the *_prev fields at that step).
-lbm_status run_resident(Engine* E, int64_t n_steps, int mom_prev) {
-  if (n_steps < 1) return LBM_OK;
-  if (n_steps >= (int64_t)1 << 30) return fail(LBM_ERR_ARG, "resident steps: at most 2^30 steps per solve");
-  if ((uint64_t)E->halo_epoch + (uint64_t)n_steps + 2 >= (1ull << 32)) {  // tags would wrap: start afresh
-    CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));
-    E->halo_epoch = 1;
-  }
-  const unsigned epoch0 = E->halo_epoch;
-  E->halo_epoch += (unsigned)n_steps + 1;
+// n_steps resident steps (moments at the last step and, when mom_prev >= 0,
+// into the *_prev fields at that step), in one launch unless there are more
+// than 2 kMaxResidentSteps; mom_prev >= n_steps - 1 - kMaxResidentSteps, so
+// that it lies in the last launch.
+constexpr int64_t kMaxResidentSteps = (int64_t)1 << 28;
+
+lbm_status run_resident(Engine* E, int64_t n_steps, int64_t mom_prev) {
   StepBarrier* bar = static_cast<StepBarrier*>(E->bar.p);
   CU(cudaMemsetAsync(&bar->error, 0, sizeof(int), E->stream));
   const int* scratch = static_cast<const int*>(E->seg_scratch.p);
-  CU(launch_stream_collide_resident(E->precision, static_cast<const LatticeView*>(E->L.views.p),
-                                    static_cast<const SegRef*>(E->segs.p), static_cast<const int*>(E->n_segs.p),
-                                    static_cast<const int*>(E->L.seg_word_off.p), scratch,
-                                    scratch + E->L.total_seg_words, E->rshape,
-                                    static_cast<unsigned long long*>(E->halo.p), E->halo_cap, epoch0, (int)n_steps,
-                                    mom_prev, &bar->error, E->stream));
+  while (n_steps > 0) {
+    const bool last = n_steps <= 2 * kMaxResidentSteps;
+    const int64_t n = last ? n_steps : kMaxResidentSteps;
+    if ((uint64_t)E->halo_epoch + (uint64_t)n + 2 >= (1ull << 32)) {  // tags would wrap: start afresh
+      CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));
+      E->halo_epoch = 1;
+    }
+    const unsigned epoch0 = E->halo_epoch;
+    E->halo_epoch += (unsigned)n + 1;
+    CU(launch_stream_collide_resident(E->precision, E->features, static_cast<const LatticeView*>(E->L.views.p),
+                                      static_cast<const SegRef*>(E->segs.p), static_cast<const int*>(E->n_segs.p),
+                                      static_cast<const int*>(E->L.seg_word_off.p), scratch,
+                                      scratch + E->L.total_seg_words, E->rshape, E->halo.p, E->halo_cap, epoch0,
+                                      (int)n, last ? (int)mom_prev : -1, &bar->error, E->stream));
+    n_steps -= n;
+    mom_prev = mom_prev < 0 ? -1 : mom_prev - n;
+  }
   E->bar_used = true;
   DEBUG_SYNC(E, "resident steps");
   return LBM_OK;
@@ -429,17 +443,16 @@ lbm_status run_resident(Engine* E, int64_t n_steps, int mom_prev) {
 
 StepConfig resident_config(const Engine* E) {
   StepConfig c{};
-  c.warps_per_block = E->rshape.warps;
+  c.warps_per_block = (E->rshape.own + 1) / 2;  // in the terms of the other shapes: two segments a warp
   c.grid = E->rshape.grid;
   c.persistent = 2;
   c.cells_per_thread = 2;
   c.stages = 0;
-  c.features = 0;
+  c.features = E->features;
   return c;
 }
 
 lbm_status run_plain_pairs(Engine* E, int64_t pairs) {
-  if (E->step.persistent == 2 && !debug_sync()) return run_resident(E, 2 * pairs, -1);
   if (E->step.persistent == 1 && !debug_sync()) return run_persistent(E, pairs);
   if (debug_sync()) {
     for (int64_t k = 0; k < pairs; ++k) {
@@ -660,15 +673,6 @@ lbm_status autotune(Engine* E) {
           cand.push_back(pairs_shape(E, wpb, scale, stages));
         }
   }
-  if (resident_enabled() && !only_plain && !E->in_group) {
-    bool ok = false;
-    lbm_status st = resident_prepare(E, &ok);
-    if (st != LBM_OK) {
-      for (void* b : backups) cudaFree(b);
-      return st;
-    }
-    if (ok) cand.push_back(resident_config(E));
-  }
   cudaEvent_t a, b;
   CU(cudaEventCreate(&a));
   CU(cudaEventCreate(&b));
@@ -681,7 +685,7 @@ lbm_status autotune(Engine* E) {
   std::vector<cudaGraphExec_t> tg(cand.size(), nullptr);
   lbm_status st = LBM_OK;
   for (size_t ci = 0; ci < cand.size() && st == LBM_OK; ++ci) {
-    if (cand[ci].persistent == 1 || cand[ci].persistent == 2) continue;  // one launch per run: no graph
+    if (cand[ci].persistent == 1) continue;  // one launch per run: no graph
     E->step = cand[ci];
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(E->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
@@ -702,9 +706,7 @@ lbm_status autotune(Engine* E) {
       const StepConfig& c = cand[ci];
       E->step = c;
       cudaEventRecord(a, E->stream);
-      if (c.persistent == 2) {
-        st = run_resident(E, 2 * kTunePairs, -1);
-      } else if (c.persistent == 1) {
+      if (c.persistent == 1) {
         st = run_persistent(E, kTunePairs);
       } else if (cudaGraphLaunch(tg[ci], E->stream) != cudaSuccess) {
         st = fail(LBM_ERR_CUDA, "autotune graph launch");
@@ -715,7 +717,7 @@ lbm_status autotune(Engine* E) {
       if (cudaEventSynchronize(b) != cudaSuccess) st = fail(LBM_ERR_CUDA, "autotune timing");
       float ms = 0.0f;
       cudaEventElapsedTime(&ms, a, b);
-      if ((c.persistent == 1 || c.persistent == 2) && st == LBM_OK) {  // a barrier that gave up would look fast: never pick it
+      if (c.persistent == 1 && st == LBM_OK) {  // a barrier that gave up would look fast: never pick it
         int err = 0;
         if (cudaMemcpy(&err, &static_cast<StepBarrier*>(E->bar.p)->error, sizeof(int), cudaMemcpyDeviceToHost) !=
             cudaSuccess)
@@ -786,8 +788,9 @@ lbm_status ensure_pinned(Engine* E, size_t n) {
   CU(cudaMallocHost((void**)&E->h_info, sizeof(int) * 8 * cap));
   CU(cudaMallocHost((void**)&E->h_count, sizeof(unsigned long long) * cap));
   CU(cudaMallocHost((void**)&E->h_nswap, sizeof(int) * cap));
-  CU(cudaMallocHost((void**)&E->h_bar_error, sizeof(int)));
+  CU(cudaMallocHost((void**)&E->h_bar_error, 2 * sizeof(int)));
   *E->h_bar_error = 0;
+  E->h_nseg = E->h_bar_error + 1;
   E->pinned_n = cap;
   return LBM_OK;
 }
@@ -983,9 +986,8 @@ Engine::~Engine() {
     for (Member* x : m) delete x;
   for (GrowBuf* b : {&L.views, &L.word_off, &L.seg_word_off, &XL.views, &XL.word_off, &XL.seg_word_off, &segs,
                      &n_segs, &seg_scratch, &partials, &result, &fluid_dev, &n_swap_dev, &dense_f, &oc_buf, &bar,
-                     &best, &rplan, &halo, &cell_list, &cell_scan, &pair_list, &pair_scan})
+                     &best, &halo, &cell_list, &cell_scan, &pair_list, &pair_scan})
     b->release();
-  if (h_rplan) cudaFreeHost(h_rplan);
   if (h_bar_error) cudaFreeHost(h_bar_error);
   if (h_result) cudaFreeHost(h_result);
   if (h_info) cudaFreeHost(h_info);
@@ -1032,7 +1034,6 @@ lbm_status engine_new(int precision, int residual_every, void* cuda_stream, bool
 }
 
 lbm_status rebuild_worklist(Engine* E) {
-  E->rplan_valid = false;
   E->cells_valid = false;
   E->pairs_valid = false;
   for (Engine* g : E->groups) {  // the groups' lists follow the members' masks
@@ -1046,6 +1047,10 @@ lbm_status rebuild_worklist(Engine* E) {
                            static_cast<int*>(E->n_segs.p), E->stream));
   CU(launch_count_fluid(static_cast<const LatticeView*>(E->L.views.p), static_cast<const int*>(E->L.word_off.p),
                         E->n(), E->L.total_words, static_cast<unsigned long long*>(E->fluid_dev.p), E->stream));
+  if (!E->in_group) {
+    CU(cudaMemcpyAsync(E->h_nseg, E->n_segs.p, sizeof(int), cudaMemcpyDeviceToHost, E->stream));
+    E->nseg_copied = true;
+  }
   DEBUG_SYNC(E, "work-list");
   return LBM_OK;
 }
@@ -1093,45 +1098,29 @@ lbm_status ensure_pairs(Engine* E) {
 
 lbm_status resident_prepare(Engine* E, bool* ok) {
   *ok = false;
-  if (E->features != 0 || E->fixed_grid || E->n() == 0 || debug_sync()) return LBM_OK;
-  if (!E->rplan_valid) {
-    NvtxRange nvtx("lbm_resident_plan");
-    CU(E->rplan.reserve(4 * sizeof(int)));
-    if (!E->h_rplan) CU(cudaMallocHost((void**)&E->h_rplan, 4 * sizeof(int)));
-    const int* scratch = static_cast<const int*>(E->seg_scratch.p);
-    CU(launch_resident_plan(static_cast<const LatticeView*>(E->L.views.p), static_cast<const SegRef*>(E->segs.p),
-                            static_cast<const int*>(E->n_segs.p), static_cast<const int*>(E->L.seg_word_off.p),
-                            scratch, scratch + E->L.total_seg_words, E->sm_count, static_cast<int*>(E->rplan.p),
-                            E->stream));
-    CU(xfer(E->h_rplan, E->rplan.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, E->stream));
+  if (E->fixed_grid || E->n() == 0 || debug_sync()) return LBM_OK;
+  if (E->nseg_copied && E->seg_bound > (long long)kResidentMaxOwn * E->sm_count) {  // the bound is too wide: count
     CU(cudaStreamSynchronize(E->stream));
-    const int nseg = E->h_rplan[0];
-    ResidentShape rs{};
-    rs.grid = resident_grid(nseg, E->sm_count);
-    const int own = (nseg + rs.grid - 1) / std::max(1, rs.grid);
-    rs.warps = std::max(1, (own + 1) / 2);
-    rs.words = E->h_rplan[1];
-    rs.pairs = E->h_rplan[2];
-    bool fits = nseg > 0 && E->h_rplan[3] == 1 && own <= kResidentMaxOwn && rs.words <= 65536 &&
-                resident_smem_bytes(E->precision, rs.words, rs.pairs) <= (size_t)std::max(0, resident_max_smem());
-    if (fits) {
-      bool moved = false;
-      const size_t bytes = (size_t)2 * nseg * 9 * 32 * sizeof(unsigned long long);
-      CU(E->halo.reserve(bytes, &moved));
-      if (moved) {  // fresh memory: no tag in it may match a future one
-        CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));
-        E->halo_epoch = 1;
-      }
-      E->halo_cap = (int)(E->halo.cap / (2 * 9 * 32 * sizeof(unsigned long long)));
-    }
-    E->rshape = rs;
-    E->rplan_ok = fits;
-    E->rplan_valid = true;
-    if (tune_log_enabled())
-      std::fprintf(stderr, "lbm resident plan: segments %d blocks %d warps %d words %d ghost rows %d fits %d\n",
-                   nseg, rs.grid, rs.warps, rs.words, rs.pairs, fits ? 1 : 0);
+    take_seg_count(E);
   }
-  *ok = E->rplan_ok;
+  const long long nseg = E->seg_bound;
+  if (nseg < 1 || nseg > (long long)kResidentMaxOwn * E->sm_count) return LBM_OK;
+  const int own = resident_own(nseg, E->sm_count);
+  E->rshape.grid = (int)((nseg + own - 1) / own);
+  const int most = (int)((nseg + E->rshape.grid - 1) / E->rshape.grid);  // segments of a block
+  E->rshape.per_warp = most <= kResidentMaxWarps ? 1 : 2;
+  E->rshape.warps = (most + E->rshape.per_warp - 1) / E->rshape.per_warp;
+  E->rshape.own = most;
+  if (E->halo_cap < nseg) {
+    // the whole word space if that is small: an exchange seldom makes the list outgrow it
+    const long long cap = std::min<long long>(E->L.total_seg_words, (long long)kResidentMaxOwn * E->sm_count);
+    bool moved = false;
+    CU(E->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap)), &moved));
+    CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));  // no tag in it may match a future one
+    E->halo_epoch = 1;
+    E->halo_cap = (int)std::max(nseg, cap);
+  }
+  *ok = true;
   return LBM_OK;
 }
 
@@ -1182,6 +1171,7 @@ lbm_status engine_set_members(Engine* E, const std::vector<Member*>& members) {
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost,
                      E->stream));
   CU(cudaStreamSynchronize(E->stream));
+  take_seg_count(E);
   for (size_t i = 0; i < n; ++i) E->m[i]->fluid_cells = (int64_t)E->h_count[i];
   return LBM_OK;
 }
@@ -1196,6 +1186,7 @@ lbm_status engine_reset(Engine* E) {
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long) * E->n(), cudaMemcpyDeviceToHost,
                      E->stream));
   CU(cudaStreamSynchronize(E->stream));
+  take_seg_count(E);
   for (int i = 0; i < E->n(); ++i) E->m[i]->fluid_cells = (int64_t)E->h_count[i];
   E->solved = false;
   return LBM_OK;
@@ -1332,10 +1323,14 @@ int engine_step_groups(const Engine* E) { return E->groups.empty() ? 1 : (int)E-
 lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
   const int K = E->residual_every;
   lbm_status st;
-  bool resident = false;
+  bool resident = E->resident_now;
   if (E->step.persistent == 2 && !debug_sync()) {
     if ((st = resident_prepare(E, &resident)) != LBM_OK) return st;
     if (!resident) E->step = shape(E, kStepWarps, kDefaultGridScale);  // the list outgrew the chip
+  }
+  if (resident && with_res && K > kMaxResidentSteps) {  // step T - K would not lie in the last launch
+    resident = false;
+    if (E->step.persistent == 2) E->step = shape(E, kStepWarps, kDefaultGridScale);
   }
   if (E->step.persistent == 3) {
     if (!cells_eligible(E)) E->step = shape(E, kStepWarps, kDefaultGridScale);
@@ -1346,7 +1341,7 @@ lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
     else if ((st = ensure_pairs(E)) != LBM_OK) return st;
   }
   if (resident) {
-    if ((st = run_resident(E, n_steps, with_res ? (int)(n_steps - K - 1) : -1)) != LBM_OK) return st;
+    if ((st = run_resident(E, n_steps, with_res ? n_steps - K - 1 : -1)) != LBM_OK) return st;
   } else if (with_res) {
     if ((st = run_plain_pairs(E, (n_steps - K) / 2 - 1)) != LBM_OK) return st;
     if ((st = launch_pair(E, 2)) != LBM_OK) return st;
@@ -1391,8 +1386,29 @@ lbm_status enqueue_steps_and_reduce(Engine* E, int64_t n_steps, bool with_res) {
   return LBM_OK;
 }
 
+// A set that fits the chip steps there, with no shape to tune, from 8 steps
+// on: a resident launch costs about as much as four per-phase steps to set up
+// and leave (solves of 16 steps, us, resident / per phase: 128 x 64 T 58 / 79,
+// 2048 x 1024 tree 108 / 138).  It is the fastest shape everywhere it fits (us
+// per step, resident / best of the others): 128 x 64 T 0.93 / 1.29, 384 x 192
+// tree 1.18 / 1.43, half-domain collector 1.22 / 2.07, 1501 x 751 tree with
+// the Smagorinsky model 1.95 / 2.52, 2048 x 1024 tree 2.02 / 3.01.
+constexpr int64_t kResidentMinSteps = 8;
+
+lbm_status choose_resident(Engine* E, int64_t n_steps) {
+  E->resident_now = false;
+  if (E->shape_fixed || !E->groups.empty() || !resident_enabled() || !autotune_enabled() ||
+      n_steps < kResidentMinSteps)
+    return LBM_OK;
+  lbm_status st = resident_prepare(E, &E->resident_now);
+  E->resident_by_rule = E->resident_now;
+  return st;
+}
+
 lbm_status enqueue_solve(Engine* E, int64_t n_steps) {
-  if (n_steps >= 256) {
+  lbm_status cst = choose_resident(E, n_steps);
+  if (cst != LBM_OK) return cst;
+  if (n_steps >= 256 && !E->resident_now) {
     lbm_status st = ensure_groups(E);
     if (st != LBM_OK) return st;
   }
@@ -1402,7 +1418,7 @@ lbm_status enqueue_solve(Engine* E, int64_t n_steps) {
         lbm_status st = autotune(g);
         if (st != LBM_OK) return st;
       }
-  } else if (!E->tuned && n_steps >= 256) {
+  } else if (!E->tuned && n_steps >= 256 && !E->resident_now) {
     lbm_status st = autotune(E);
     if (st != LBM_OK) return st;
   }
@@ -1439,6 +1455,8 @@ lbm_status enqueue_exchange(Engine* E, const std::vector<int>& which, const int3
     Member* m = E->m[i];
     if (m->p.reinit == LBM_REINIT_COLD) CU(cudaMemsetAsync(m->f, 0, 9 * m->plane * sb, E->stream));
   }
+  for (int k = 0; k < nx_; ++k) E->seg_bound += n_swap[k];  // a new fluid cell opens at most one segment
+  E->seg_bound = std::min<long long>(E->seg_bound, E->L.total_seg_words);
   st = rebuild_worklist(E);
   if (st != LBM_OK) return st;
   CU(xfer(E->h_info, E->oc.info, sizeof(int) * 8 * nx_, cudaMemcpyDeviceToHost, E->stream));
@@ -1499,6 +1517,7 @@ lbm_status engine_solve(Engine* E, int64_t n_steps, lbm_solve_result* out) {
   lbm_status st = enqueue_solve(E, n_steps);
   if (st != LBM_OK) return st;
   CU(cudaStreamSynchronize(E->stream));
+  take_seg_count(E);
   for (Member* m : E->m) m->steps_done += n_steps;
   E->solved = true;
   account_steps(E, n_steps);
@@ -1527,6 +1546,7 @@ lbm_status engine_optimize(Engine* E, const int32_t* n_swap, int64_t n_steps, lb
   st = enqueue_solve(E, n_steps);
   if (st != LBM_OK) return st;
   CU(cudaStreamSynchronize(E->stream));
+  take_seg_count(E);
   bool nan = false, count_changed = false, bad = false;
   for (int i = 0; i < E->n(); ++i) {
     Member* m = E->m[i];
@@ -1585,6 +1605,7 @@ lbm_status restore_state(Engine* E, Member* m) {
   if (st != LBM_OK) return st;
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long), cudaMemcpyDeviceToHost, E->stream));
   CU(cudaStreamSynchronize(E->stream));
+  take_seg_count(E);
   m->fluid_cells = (int64_t)E->h_count[0];
   return LBM_OK;
 }
@@ -1682,7 +1703,12 @@ lbm_status engine_read(Engine* E, int i, uint32_t which, void* dst, size_t dst_b
 
 lbm_status engine_step_config(Engine* E, int32_t* warps_per_block, int32_t* grid, int32_t* persistent,
                               int32_t* cells_per_thread, int32_t* stages) {
-  const StepConfig& c = E->groups.empty() ? E->step : E->groups[0]->step;  // grouped: the first group's
+  // grouped: the first group's; a plain lattice on the chip by rule: that
+  // shape (batches and lattices with features report the per-phase shape that
+  // their short solves take)
+  const StepConfig c = !E->groups.empty()                                             ? E->groups[0]->step
+                       : E->resident_by_rule && E->features == 0 && E->n() == 1 ? resident_config(E)
+                                                                                : E->step;
   if (warps_per_block) *warps_per_block = c.warps_per_block;
   if (grid) *grid = c.grid;
   if (persistent) *persistent = c.persistent;
@@ -1695,12 +1721,13 @@ lbm_status engine_set_step_config(Engine* E, int32_t warps_per_block, int32_t pe
                                   int32_t stages) {
   // a fixed shape applies to the whole set: no member groups
   E->shape_fixed = true;
+  E->resident_now = E->resident_by_rule = false;
   E->groups_decided = true;
   for (Engine* g : E->groups) delete g;
   E->groups.clear();
   if (persistent == 2) {  // on-chip resident steps: the shape follows from the work-list
     bool ok = false;
-    lbm_status st = resident_prepare(E, &ok);
+    lbm_status st = E->features ? LBM_OK : resident_prepare(E, &ok);
     if (st != LBM_OK) return st;
     if (!ok)
       return fail(LBM_ERR_ARG, "resident steps need plain BGK lattices whose segments fit in shared memory");

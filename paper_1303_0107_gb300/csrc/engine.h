@@ -116,12 +116,16 @@ struct Engine {
   int* h_bar_error = nullptr;             // pinned: grid-barrier error flag of the last solve
   bool bar_used = false;                  // the last enqueued solve ran the persistent kernel
 
-  // on-chip resident steps (step.persistent == 2): the plan of the current
-  // work-list (valid until the list is rebuilt), the halo buffer of tagged
+  // on-chip resident steps (step.persistent == 2): a host-side bound on the
+  // segments of the current work-list (exact when the list was last counted,
+  // then raised by what each exchange can add), the halo buffer of tagged
   // words and the next tag
-  GrowBuf rplan, halo;
-  int* h_rplan = nullptr;  // pinned [4]
-  bool rplan_valid = false, rplan_ok = false;
+  long long seg_bound = 0;
+  int* h_nseg = nullptr;   // pinned: the list's count, copied after a rebuild
+  bool nseg_copied = false;
+  bool resident_now = false;      // the solve being enqueued steps on the chip by rule
+  bool resident_by_rule = false;  // so did the last one long enough for the rule
+  GrowBuf halo;
   ResidentShape rshape{};
   int halo_cap = 0;        // segments the halo buffer holds
   unsigned halo_epoch = 1;
@@ -171,8 +175,8 @@ lbm_status engine_reset(Engine* E);
 // Number of member groups the time steps run in (1 when not grouped).
 int engine_step_groups(const Engine* E);
 lbm_status rebuild_worklist(Engine* E);
-// Plan the resident launch for the current work-list (synchronises the
-// stream when the list changed since the last plan); *ok: the set fits.
+// Shape and halo buffer of a resident launch over the current work-list;
+// *ok: the set fits the chip.
 lbm_status resident_prepare(Engine* E, bool* ok);
 // Compacted fluid-cell tasks: whether the set may use them (plain BGK, no
 // zero-gradient outlet), and the list built for the current work-list.

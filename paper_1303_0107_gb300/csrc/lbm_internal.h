@@ -199,43 +199,42 @@ int stream_collide_persistent_grid(int precision, int warps_per_block, int cells
 // ---- on-chip resident time steps (resident.cu) ------------------------------
 // A whole solve in one cooperative launch with the populations in shared
 // memory: block b of G owns segments [b n / G, (b+1) n / G) of the list
-// (at most kResidentMaxOwn), two per warp, and exchanges the rows its
-// neighbours need through a halo buffer of tagged words.
+// (at most kResidentMaxOwn), one or two per warp, and exchanges what its neighbours
+// need through a halo buffer of tagged words.
 constexpr int kResidentMaxOwn = 48;
-constexpr int kResidentMaxWarps = kResidentMaxOwn / 2;
-// blocks of a resident launch over n segments: as few as hold them, at most one per SM
-__host__ __device__ inline int resident_grid(int nseg, int sm_count) {
-  const int need = (nseg + kResidentMaxOwn - 1) / kResidentMaxOwn;
-  return need < 1 ? 1 : need > sm_count ? sm_count : need;
+constexpr int kResidentMaxWarps = 32;
+// Segments per block of a resident launch over nseg: an equal share of every
+// SM, in whole groups of four, but not below 16 -- a step of a small list is
+// the chain from one block's published words to its neighbours' update, which
+// more blocks do not shorten.  Measured, us per step at 32 / 20 / 16 / 12 / 8
+// segments a block: 88 segments (128 x 64 T) 1.19 / 1.03 / 0.93 / 1.07 / 1.07;
+// 414 (384 x 192 tree) 1.25 / 1.19 / 1.18 / 1.04 / 1.15; 1178 (collector)
+// 1.47 / 1.29 / 1.22 / 1.14 / 1.17; 6976 (2048 x 1024 tree) at 48 and 46:
+// 2.02 / 1.98.
+__host__ __device__ inline int resident_own(long long nseg, int sm_count) {
+  const long long share = ((nseg + sm_count - 1) / sm_count + 3) / 4 * 4;
+  return share < 16 ? 16 : share > kResidentMaxOwn ? kResidentMaxOwn : (int)share;
 }
-// elements between the two step buffers: words rounded up to 8, a multiple
-// of 16 bytes for 16-bit and 32-bit storage
-__host__ __device__ inline int resident_buffer_stride(int words) { return (words + 7) & ~7; }
 struct ResidentShape {
-  int grid;   // blocks
-  int warps;  // warps per block (two segments each)
-  int words;  // step-buffer size per block (elements of the storage type)
-  int pairs;  // ghost rows per block at most
+  int grid;      // blocks
+  int warps;     // warps per block
+  int per_warp;  // segments per warp, 1 or 2
+  int own;       // segments of the fullest block
 };
-// Plan for the current list (out: int[4], device): segments, largest
-// step-buffer size, largest ghost-row count, 1 if the list fits.  seg_flags /
-// seg_offs: the work-list build's per-word flags and their exclusive scan
-// (the list index of every segment word that holds fluid).
-cudaError_t launch_resident_plan(const LatticeView* views, const SegRef* segs, const int* n_segs,
-                                 const int* seg_word_off, const int* seg_flags, const int* seg_offs, int sm_count,
-                                 int* out, cudaStream_t stream);
-// Dynamic shared memory of a launch, and the most a block may take.
-size_t resident_smem_bytes(int precision, int words, int pairs);
-int resident_max_smem();
-// n_steps time steps; halo: [2][halo_cap][9][32] words of {value, tag}, tags
-// epoch0 + 1 .. epoch0 + n_steps - 1 written by this launch (older tags
+// Bytes of a halo buffer for a list of that many segments.
+size_t resident_halo_bytes(int segments);
+// n_steps (even) time steps of a list of at most rs.per_warp rs.warps rs.grid segments;
+// features: kernel build as in StepConfig; seg_flags / seg_offs: the
+// work-list build's per-word flags and their exclusive scan (the list index
+// of every segment word that holds fluid); halo: room for halo_cap segments,
+// tags epoch0 + 1 .. epoch0 + n_steps - 1 written by this launch (older tags
 // must all be smaller); moments at the last step and at step mom_prev (-1:
 // none, else into the *_prev fields); *error is set when a wait gave up.
-cudaError_t launch_stream_collide_resident(int precision, const LatticeView* views, const SegRef* segs,
+cudaError_t launch_stream_collide_resident(int precision, int features, const LatticeView* views, const SegRef* segs,
                                            const int* n_segs, const int* seg_word_off, const int* seg_flags,
-                                           const int* seg_offs, const ResidentShape& rs,
-                                           unsigned long long* halo, int halo_cap, unsigned epoch0, int n_steps,
-                                           int mom_prev, int* error, cudaStream_t stream);
+                                           const int* seg_offs, const ResidentShape& rs, void* halo, int halo_cap,
+                                           unsigned epoch0, int n_steps, int mom_prev, int* error,
+                                           cudaStream_t stream);
 
 // ---- geometry / work-list (worklist.cu) ------------------------------------
 cudaError_t launch_pack_mask(const uint8_t* cells, int nx, int ny, int wpr, uint32_t* mask,

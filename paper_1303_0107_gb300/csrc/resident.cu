@@ -2,49 +2,93 @@
 // held in shared memory from its first step to its last.
 //
 // Method: the same per-cell update as the step kernels (Eq. 1 with the
-// equilibrium of Sec. 2.1, the moments of Eq. 2, halfway bounce-back and the
-// port rules of Sec. 3.3; d2q9_cell.cuh), so every cell gets the same bits.
+// equilibrium of Sec. 2.1, the moments of Eq. 2, halfway bounce-back, the
+// port rules and the symmetry plane of Sec. 3.3; d2q9_cell.cuh), so every
+// cell gets the same bits.
 //
 // Layout.  A lattice set whose row segments fit in the shared memory of the
 // SMs (the 2048 x 1024 distributor: 6976 segments, 5.75 MB of FP32
 // populations, against 152 x 227 KB) is split into contiguous ranges of its
 // segment list, one range per block (at most kResidentMaxOwn segments, one
 // block per SM, all blocks resident: a cooperative launch).  A block keeps
-// its segments' nine population rows in two step buffers in shared memory
-// (read one, write the other, a plain pull scheme), plus copies of the
-// population rows it needs from segments of other blocks ("ghosts": per
-// neighbouring segment only the directions that stream across, e.g. the
-// three upward directions of the segment below).
+// its segments' nine population rows as FP32 in two step buffers in shared
+// memory (read one, write the other, a plain pull scheme; 16-bit storage
+// rounds every value to its type before it is stored, so the values are
+// those of 16-bit buffers without their conversions on every load).
 //
-// Exchange.  After each step a block publishes, for each of its segments
-// that another block reads, the directions that block needs, as 64-bit words
-// {value, step tag} in a halo buffer in global memory (two step parities).
-// Before the next step it polls the words of its ghosts until each carries
-// the expected tag: value and tag travel in one single-copy-atomic word, so
-// there is no fence and no flag, and a block waits only for its neighbours
-// -- no grid-wide barrier.  Two parities suffice: a block can overwrite a
-// word of step t only after it has read its neighbours' step t + 1 words,
-// which they publish after reading its step t words.  Every wait is bounded:
-// a block that gives up sets the error word and leaves, and the others leave
-// at their next check of that word.
+// Thread mapping.  A warp owns one segment, lane l its cell l; lists of more
+// than 32 segments per SM (the register budget of 1024 threads) take two per
+// warp, collided as one in the packed FP32 instructions (bgk2).  One is the
+// better mapping where it fits: a step is a chain of dependent stages (words
+// arrive, pull, ports, collision, publish), and with two segments each stage
+// is twice as long (20 segments a block, 1024 x 512 tree: 1.26 us per step
+// against 1.56).  Each lane knows, for its cell and eight directions, the
+// shared-memory word its incoming value comes from, computed once per launch:
+// an own row, another slot's row, a ghost word, its own opposite slot
+// (bounce-back), or a word that stays zero (the unknown populations of port
+// cells; every direction of a solid cell).  No step branches on the geometry.
 //
-// Per step and block: fetch the ghosts, one __syncthreads, then each warp
-// updates its (at most two) segments -- the published ones first, so that
-// neighbours can proceed while the rest is computed -- pulling from the
-// current buffer through source offsets computed once per launch (own row,
-// neighbouring own segment, ghost row, bounce-back into the cell's own slot,
-// or a zero word for the unknown populations of port cells).  The lattice
-// is read from the canonical global layout at the start of the launch and
-// written back to it at the end.
+// Exchange.  After each step a warp publishes, for each of its segments
+// that another block reads, 16-byte words {value, value, value, step tag}:
+// what streams up (directions 2, 5, 6), what streams down (4, 7, 8) and, for
+// the segments beside it, what streams sideways (1, 3).  One word per lane
+// carries all that the segment above or below needs of that lane, and value
+// and tag travel in one single-copy-atomic 128-bit access, so there is no
+// fence and no flag.  Before the next step the warp that owns a reading
+// segment polls the words it needs -- a row per vertical neighbour, single
+// words at the corners and sides -- into ghost words of its own.  Nothing
+// but the block's own barrier orders the warps of a block: a warp whose
+// segments touch no other block computes while the others wait for their
+// words.  Two parities suffice: a warp overwrites a word of step t only
+// after it has read its neighbour's word of step t + 1 (reading is mutual),
+// which that neighbour publishes after reading the word of step t.  Every
+// wait is bounded: a warp that gives up makes its block set the error word
+// and leave, and the others leave when they see it.
+//
+// What bounds it.  The exchange costs 500 to 720 cycles through L2 between
+// SMs of one die and about 1050 between dies; the rest of a lone warp's step
+// about 700, and 300 to 400 more where it holds a port cell.  Small lists run
+// at that chain: 0.93 us per step (128 x 64 T, 88 segments; 1.31 us before, one
+// launch per phase).  The 2048 x 1024 tree (46-48 segments a block) adds the
+// issue of 24 packed pairs, 330 warp instructions each: 2.02 us per step, 2.27
+// before (ghost rows fetched by the whole block before a barrier, one cell a
+// lane, one 64-bit word per value); with BF16 storage 2.14, 2.64 before.
+// Barriers between the warps that share segments instead of the block's (one
+// mbarrier per warp and parity) ran 2.20; two segments per warp one after the
+// other 2.39; a spilled register costs an L2 round trip here, because shared
+// memory leaves the L1 cache next to nothing.
 #include "d2q9_cell.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int kSegWords = 9 * 32;  // one segment's populations in a step buffer
 constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned kResidentSpinLimit = 1u << 22;
-constexpr int kFetch = 6;  // ghost rows a warp keeps in flight
+constexpr int kFeatModels = 1, kFeatMirror = 2;  // kernel builds, as in step.cu
+
+// A step buffer in shared memory, in 4-byte words: the own rows of every
+// slot ([9][32] each), then the ghost words of every slot, then a zero word.
+// Ghost words of a slot: six rows of 34 (the word of lane l at 1 + l, the
+// corner segments' at 0 and 33), rows 0-2 directions 4, 7, 8 from above,
+// rows 3-5 directions 2, 5, 6 from below, then the side segments' words
+// (direction 1 from the west, 3 from the east).
+constexpr int kSegWords = 9 * 32;
+constexpr int kGhostRow = 34;
+constexpr int kGhostWest = 6 * kGhostRow, kGhostEast = kGhostWest + 1;
+constexpr int kGhostWords = kGhostEast + 1;
+template <int S>  // segments per warp
+struct Layout {
+  static constexpr int kWarps = S == 1 ? kResidentMaxWarps : kResidentMaxOwn / 2;
+  static constexpr int kSlots = S * kWarps;
+  static constexpr int kGhost0 = kSlots * kSegWords;
+  static constexpr int kZero = kGhost0 + kSlots * kGhostWords;
+  static constexpr int kWords = (kZero + 4) & ~3;
+  static_assert(kWords <= 65536, "two slots' source words share a register");
+};
+
+// Published words of a segment, 16 bytes each: [unit][lane]
+constexpr int kUnitUp = 0, kUnitDown = 1, kUnitSide = 2;
+constexpr int kUnitWords = 32;
 
 // Neighbouring segments of (y, w), position p = 0..7: E N W S NE NW SW SE,
 // (dy, dw) = (0,1) (1,0) (0,-1) (-1,0) (1,1) (1,-1) (-1,-1) (-1,1).
@@ -57,51 +101,58 @@ __device__ __forceinline__ int pos_of(int dy, int dw) {
   if (dy > 0) return dw > 0 ? 4 : 5;
   return dw < 0 ? 6 : 7;
 }
-// Directions a cell pulls from the segment at position p (bit i = direction
-// i): from the segment above the three with c_y = -1, from the one below the
-// three with c_y = +1, from a side or corner segment only the one direction
-// that reaches its edge lane.
-__device__ __forceinline__ unsigned need_mask(int p) {
-  switch (p) {
-    case 0: return 1u << 3;                            // E: W-moving
-    case 1: return (1u << 4) | (1u << 7) | (1u << 8);  // N: S, SW, SE
-    case 2: return 1u << 1;                            // W: E-moving
-    case 3: return (1u << 2) | (1u << 5) | (1u << 6);  // S: N, NE, NW
-    case 4: return 1u << 7;                            // NE: SW
-    case 5: return 1u << 8;                            // NW: SE
-    case 6: return 1u << 5;                            // SW: NE
-    default: return 1u << 6;                           // SE: NW
-  }
-}
-__device__ __forceinline__ int opp_pos(int p) { return p ^ 2; }
 
 // D2Q9 velocities and opposites (compile-time indices after unrolling)
 __host__ __device__ constexpr int cx_of(int i) { return i == 1 || i == 5 || i == 8 ? 1 : i == 3 || i == 6 || i == 7 ? -1 : 0; }
 __host__ __device__ constexpr int cy_of(int i) { return i == 2 || i == 5 || i == 6 ? 1 : i == 4 || i == 7 || i == 8 ? -1 : 0; }
 __host__ __device__ constexpr int opp_of(int i) { return i == 0 ? 0 : i <= 4 ? ((i + 1) & 3) + 1 : ((i - 5 + 2) & 3) + 5; }
+// ghost row of direction i arriving from above (4, 7, 8) or below (2, 5, 6)
+__host__ __device__ constexpr int ghost_row(int i) {
+  return i == 4 ? 0 : i == 7 ? 1 : i == 8 ? 2 : i == 2 ? 3 : i == 5 ? 4 : 5;
+}
 
+// Both values to the storage type and back (round to nearest even).
 template <class T>
-__device__ __forceinline__ float round_to_storage(float v);
+__device__ __forceinline__ void round2(float& a, float& b);
 template <>
-__device__ __forceinline__ float round_to_storage<float>(float v) { return v; }
+__device__ __forceinline__ void round2<float>(float&, float&) {}  // (the two may be one and the same)
 template <>
-__device__ __forceinline__ float round_to_storage<__nv_bfloat16>(float v) {
-  return __bfloat162float(__float2bfloat16_rn(v));
+__device__ __forceinline__ void round2<__nv_bfloat16>(float& a, float& b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  a = __low2float(h);
+  b = __high2float(h);
 }
 template <>
-__device__ __forceinline__ float round_to_storage<__half>(float v) { return __half2float(__float2half_rn(v)); }
+__device__ __forceinline__ void round2<__half>(float& a, float& b) {
+  const float2 v = __half22float2(__floats2half2_rn(a, b));
+  a = v.x;
+  b = v.y;
+}
 
-// Relaxed (L2-coherent) accesses of the halo words and the error word.  No
-// memory clobber: each poll's use of its value orders it, and the compiler
-// may keep the launch-constant descriptor fields in registers across them.
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p));
+// A published word: three values and the step tag, one 128-bit access
+// (relaxed, GPU scope: coherent in L2).  No memory clobber: each poll's use
+// of its value orders it.
+struct HaloWord {
+  unsigned long long lo, hi;  // lo: values 0 and 1; hi: value 2 and the tag
+};
+__device__ __forceinline__ HaloWord halo_ld(const HaloWord* p) {
+  HaloWord v;
+  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+               : "=l"(v.lo), "=l"(v.hi)
+               : "l"(p));
   return v;
 }
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v));
+__device__ __forceinline__ void halo_st(HaloWord* p, float v0, float v1, float v2, unsigned tag) {
+  const unsigned long long lo = (unsigned long long)__float_as_uint(v1) << 32 | __float_as_uint(v0);
+  const unsigned long long hi = (unsigned long long)tag << 32 | __float_as_uint(v2);
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+               "l"(lo), "l"(hi));
 }
+__device__ __forceinline__ float halo_value(const HaloWord& w, int k) {
+  return __uint_as_float(k == 0 ? (unsigned)w.lo : k == 1 ? (unsigned)(w.lo >> 32) : (unsigned)w.hi);
+}
+__device__ __forceinline__ unsigned halo_tag(const HaloWord& w) { return (unsigned)(w.hi >> 32); }
+
 __device__ __forceinline__ int ld_relaxed_s32(const int* p) {
   int v;
   asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
@@ -120,210 +171,284 @@ __device__ __forceinline__ int list_index(const LatticeView* __restrict__ views,
   return seg_flags[i] ? seg_offs[i] : -1;
 }
 
-// What a block knows about its own segments (t: position in its range).
-struct OwnInfo {
-  int nbq[kResidentMaxOwn][8];  // list index of each neighbouring segment, or -1
-  unsigned pub[kResidentMaxOwn];  // directions other blocks read from segment t
-  int npairs[kResidentMaxOwn];    // ghost rows segment t needs
-  unsigned remote[kResidentMaxOwn];  // bit p: the neighbour at position p belongs to another block
-};
-
-// Fill `oi` for the block's range [s0, s1) (every thread of the block calls).
-__device__ void describe_range(const LatticeView* __restrict__ views, const SegRef* __restrict__ segs,
-                               const int* __restrict__ seg_word_off, const int* __restrict__ seg_flags,
-                               const int* __restrict__ seg_offs, int s0, int s1, OwnInfo& oi) {
-  for (int t = threadIdx.x; t < s1 - s0; t += blockDim.x) {
-    const SegRef sr = segs[s0 + t];
-    const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
-    unsigned pub = 0, rem = 0;
-    int np = 0;
-    for (int p = 0; p < 8; ++p) {
-      const int nq = list_index(views, seg_word_off, seg_flags, seg_offs, sr.lattice, y + pos_dy(p), w + pos_dw(p));
-      oi.nbq[t][p] = nq;
-      if (nq >= 0 && (nq < s0 || nq >= s1)) {
-        rem |= 1u << p;
-        pub |= need_mask(opp_pos(p));
-        np += __popc(need_mask(p));
-      }
-    }
-    oi.pub[t] = pub;
-    oi.remote[t] = rem;
-    oi.npairs[t] = np;
-  }
-}
-
 __device__ __forceinline__ void block_range(int nseg, int G, int b, int& s0, int& s1) {
   s0 = (int)((long long)b * nseg / G);
   s1 = (int)((long long)(b + 1) * nseg / G);
 }
 
-// The block's ghost rows: the (segment, direction) keys (segment << 4 |
-// direction) its segments pull from other blocks, each once, ascending, into
-// out; returns their number.  raw and first: scratch of 12 n_own ints each
-// (a segment needs at most 3 + 3 + 1 + 1 + 4 x 1 rows).  Every thread calls.
-__device__ int collect_ghosts(const OwnInfo& oi, int n_own, int* raw, int* first, int* out) {
-  __shared__ int s_base[kResidentMaxOwn + 1];
-  __shared__ int s_unique;
-  if (threadIdx.x == 0) {
-    int b = 0;
-    for (int t = 0; t < n_own; ++t) {
-      s_base[t] = b;
-      b += oi.npairs[t];
+// slot flags
+constexpr unsigned kPubUp = 1u, kPubDown = 2u, kPubSide = 4u, kHasPort = 8u, kNeumann = 16u, kSlotModel = 32u;
+constexpr unsigned kPublishes = kPubUp | kPubDown | kPubSide;
+
+// What a step seldom needs of a slot, in shared memory.
+struct alignas(16) SlotInfo {
+  int in_lane, out_lane; // lanes of its inlet and outlet cell, -1: none
+  float u_in;            // inlet speed of its row
+  int zou_he;            // port scheme
+  long long row;         // element offset of the segment's first cell in its lattice
+  const LatticeView* L;
+  unsigned fluid;        // its fluid lanes
+};
+struct alignas(16) PairInfo {  // of a warp's two slots
+  float rho0[2], omega[2];
+  unsigned flags;  // slot flags: slot 2w in the low half, 2w + 1 in the high
+  int unit0[2];    // first published word of each slot, (list index * 3) * 32
+  int pad;
+  int vert[4];    // words of the segments above and below slot 0, then slot 1; -1: none remote
+  int edge[16];   // lanes 0-5 (slot 0) and 8-13 (slot 1): (word << 2 | value) of W E NW NE SW SE; -1: none
+};
+
+// Fetch this warp's ghost words of step k into buffer `buf`; false: gave up.
+template <int S>
+__device__ __forceinline__ bool fetch_ghosts(float* buf, const PairInfo& pi, const HaloWord* halo, int parity,
+                                             unsigned want, int lane, int* error) {
+  const HaloWord* hb = halo + parity;
+  const int4 vt = *reinterpret_cast<const int4*>(pi.vert);
+  const int es = lane < 8 * S ? pi.edge[lane] : -1;
+  HaloWord v[2 * S], e;
+  const unsigned long long ready = (unsigned long long)want << 32;
+  const int src[4] = {vt.x, vt.y, vt.z, vt.w};
+#pragma unroll
+  for (int u = 0; u < 2 * S; ++u) {
+    v[u].hi = ready;
+    if (src[u] >= 0) v[u] = halo_ld(hb + src[u] + lane);  // warp-uniform
+  }
+  e.hi = ready;
+  if (es >= 0) e = halo_ld(hb + (es >> 2));
+  unsigned spins = 0;
+  for (;;) {
+    bool ok = halo_tag(e) == want;
+#pragma unroll
+    for (int u = 0; u < 2 * S; ++u) ok &= halo_tag(v[u]) == want;
+    if (__all_sync(kFull, ok)) break;
+#pragma unroll
+    for (int u = 0; u < 2 * S; ++u)
+      if (halo_tag(v[u]) != want) v[u] = halo_ld(hb + src[u] + lane);
+    if (halo_tag(e) != want) e = halo_ld(hb + (es >> 2));
+    ++spins;
+    if (spins > kResidentSpinLimit || ((spins & 255u) == 0 && __any_sync(kFull, ld_relaxed_s32(error) != 0))) {
+      if (lane == 0) atomicExch(error, 1);
+      return false;
     }
-    s_base[n_own] = b;
   }
-  __syncthreads();
-  for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
-    int k = s_base[t];
-    for (int p = 0; p < 8; ++p) {
-      if (!((oi.remote[t] >> p) & 1u)) continue;
-      const unsigned m = need_mask(p);
-      for (int i = 1; i <= 8; ++i)
-        if ((m >> i) & 1u) raw[k++] = (oi.nbq[t][p] << 4) | i;
+  float* ga = buf + Layout<S>::kGhost0 + S * (threadIdx.x >> 5) * kGhostWords;
+#pragma unroll
+  for (int u = 0; u < 2 * S; ++u)
+    if (src[u] >= 0) {
+      float* g = ga + (u >> 1) * kGhostWords + (u & 1) * 3 * kGhostRow + 1 + lane;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) g[d * kGhostRow] = halo_value(v[u], d);
     }
+  if (es >= 0) {
+    const int item = lane & 7;
+    const int at = item == 0 ? kGhostWest : item == 1 ? kGhostEast : item == 2 ? 2 * kGhostRow
+                 : item == 3 ? 1 * kGhostRow + 33 : item == 4 ? 4 * kGhostRow : 5 * kGhostRow + 33;
+    ga[(lane >> 3) * kGhostWords + at] = halo_value(e, es & 3);
   }
-  __syncthreads();
-  const int n = s_base[n_own];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {  // first occurrence of each key
-    int f = 1;
-    for (int j = 0; j < i && f; ++j) f = raw[j] != raw[i];
-    first[i] = f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    if (first[i]) {
-      int pos = 0;
-      for (int j = 0; j < n; ++j) pos += first[j] && raw[j] < raw[i];
-      out[pos] = raw[i];
-    }
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int j = 0; j < n; ++j) c += first[j];
-    s_unique = c;
-  }
-  __syncthreads();
-  return s_unique;
+  __syncwarp();
+  return true;
 }
 
-// Position of key in the ascending out[0 .. n), or -1.
-__device__ __forceinline__ int find_ghost(const int* out, int n, int key) {
-  int lo = 0, hi = n - 1;
-  while (lo <= hi) {
-    const int mid = (lo + hi) >> 1;
-    const int v = out[mid];
-    if (v == key) return mid;
-    if (v < key) lo = mid + 1; else hi = mid - 1;
+// Port rules of the slot's port cells (all lanes call).
+__device__ __forceinline__ void ports_of(float (&g)[9], unsigned slot_flags, const SlotInfo& si, float rho0, int lane) {
+  const int4 pw = *reinterpret_cast<const int4*>(&si);  // in_lane, out_lane, u_in, zou_he
+  const bool out = lane == pw.y;
+  if (slot_flags & kNeumann) {  // zero-gradient outlet: cell nx-2 is the lane to the left
+    const float n3 = __shfl_up_sync(kFull, g[3], 1);
+    const float n6 = __shfl_up_sync(kFull, g[6], 1);
+    const float n7 = __shfl_up_sync(kFull, g[7], 1);
+    if (out) {
+      g[3] = n3;
+      g[6] = n6;
+      g[7] = n7;
+    }
   }
-  return -1;
+  const int scheme = pw.w ? LBM_PORTS_ZOU_HE : LBM_PORTS_REGULARIZED;
+  if (lane == pw.x)
+    inlet_rule(g, __int_as_float(pw.z), rho0, scheme);
+  else if (out && !(slot_flags & kNeumann))
+    outlet_rule(g, rho0, scheme);
 }
 
-// Plan of a resident launch for the current segment list: out[0] = segments,
-// out[1] = largest step-buffer size of any block (words of the storage
-// type), out[2] = largest ghost-row count, out[3] = 1 if every block's range
-// fits kResidentMaxOwn.  out must be zeroed first.
-__global__ void k_resident_plan(const LatticeView* __restrict__ views, const SegRef* __restrict__ segs,
-                                const int* __restrict__ n_segs, const int* __restrict__ seg_word_off,
-                                const int* __restrict__ seg_flags, const int* __restrict__ seg_offs, int sm_count,
-                                int* __restrict__ out) {
-  __shared__ OwnInfo oi;
-  __shared__ int raw[12 * kResidentMaxOwn], first[12 * kResidentMaxOwn], uniq[12 * kResidentMaxOwn];
-  const int nseg = n_segs[0];
-  const int G = resident_grid(nseg, sm_count);
-  if (blockIdx.x >= G) return;
-  int s0, s1;
-  block_range(nseg, G, blockIdx.x, s0, s1);
-  if (s1 - s0 > kResidentMaxOwn) {  // the whole list does not fit on the device
-    if (threadIdx.x == 0) atomicMax(out + 0, nseg);
-    return;
+__device__ __forceinline__ void write_moments(const SlotInfo& si, int lane, bool last, float drho, float ux, float uy) {
+  const LatticeView& L = *si.L;
+  const long long c = si.row + lane;
+  L.drho[c] = drho;
+  (last ? L.ux : L.ux_prev)[c] = ux;
+  (last ? L.uy : L.uy_prev)[c] = uy;
+}
+
+// hb: this lane's word of the segment's first unit
+__device__ __forceinline__ void publish(HaloWord* hb, unsigned flags, int lane, const float (&g)[9], unsigned tag) {
+  if (flags & kPubUp) halo_st(hb + kUnitUp * kUnitWords, g[2], g[5], g[6], tag);
+  if (flags & kPubDown) halo_st(hb + kUnitDown * kUnitWords, g[4], g[7], g[8], tag);
+  if ((flags & kPubSide) && (lane == 0 || lane == 31)) halo_st(hb + kUnitSide * kUnitWords, g[1], g[3], 0.0f, tag);
+}
+
+// One time step of the warp's S segments: buffer PAR read, the other written.
+template <class T, int FEAT, int S, int PAR>
+__device__ __forceinline__ void warp_step(float* sm, const unsigned (&off)[8], unsigned own, int k, int k_last,
+                                          int mom_prev, unsigned epoch0, const PairInfo& pi, const SlotInfo* si,
+                                          HaloWord* halo, int parity, int lane) {
+  constexpr int kCur = PAR * Layout<S>::kWords, kNxt = (PAR ^ 1) * Layout<S>::kWords;
+  float g[S][9];
+#pragma unroll
+  for (int r = 0; r < S; ++r) g[r][0] = sm[own + r * kSegWords + kCur];
+#pragma unroll
+  for (int i = 1; i <= 8; ++i) {
+    unsigned o = off[i - 1];
+    if (S == 2) asm volatile("" : "+r"(o));  // unpacked here, at every step: hoisted, the sixteen words spill
+    g[0][i] = sm[(S == 2 ? o & 0xffffu : o) + kCur];
+    if (S == 2) g[S - 1][i] = sm[(o >> 16) + kCur];
   }
-  __syncthreads();
-  describe_range(views, segs, seg_word_off, seg_flags, seg_offs, s0, s1, oi);
-  __syncthreads();
-  const int np = collect_ghosts(oi, s1 - s0, raw, first, uniq);
-  if (threadIdx.x == 0) {
-    atomicMax(out + 0, nseg);
-    atomicMax(out + 1, (s1 - s0) * kSegWords + np * 32 + 1);
-    atomicMax(out + 2, np);
-    if (blockIdx.x == 0) atomicMax(out + 3, (int)(((long long)nseg + G - 1) / G <= kResidentMaxOwn));
+  const float4 par = *reinterpret_cast<const float4*>(pi.rho0);  // rho0 and omega of the slots
+  const int4 units = *reinterpret_cast<const int4*>(&pi.flags);
+  const unsigned flags = (unsigned)units.x;
+  if (flags & (kHasPort << 16 | kHasPort)) {  // warp-uniform
+    if (flags & kHasPort) ports_of(g[0], flags, si[0], par.x, lane);
+    if (S == 2 && (flags & kHasPort << 16)) ports_of(g[S - 1], flags >> 16, si[S - 1], par.y, lane);
+  }
+  float dr[S], ux[S], uy[S];
+  const bool models = (FEAT & kFeatModels) && (flags & (kSlotModel << 16 | kSlotModel));
+  if (models || S == 1) {
+#pragma unroll
+    for (int r = 0; r < S; ++r) {
+      const float rho0 = r ? par.y : par.x, omega = r ? par.w : par.z;
+      if (models && (flags & kSlotModel << (16 * r)))
+        collide_other(g[r], rho0, omega, si[r].L->collision, si[r].L->c_smag, dr[r], ux[r], uy[r]);
+      else
+        bgk(g[r], rho0, omega, dr[r], ux[r], uy[r]);
+    }
+  } else {
+    bgk2(g[0], g[S - 1], f2(par.x, par.y), f2(par.z, par.w), dr[0], ux[0], uy[0], dr[S - 1], ux[S - 1], uy[S - 1]);
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) round2<T>(g[0][i], g[S - 1][i]);
+  if ((flags & (kPublishes << 16 | kPublishes)) && k != k_last) {
+    const unsigned tag = epoch0 + (unsigned)k + 1u;
+    HaloWord* hb = halo + (parity + lane);
+    if (flags & kPublishes) publish(hb + units.y, flags, lane, g[0], tag);
+    if (S == 2 && (flags & kPublishes << 16)) publish(hb + units.z, flags >> 16, lane, g[S - 1], tag);
+  }
+#pragma unroll
+  for (int r = 0; r < S; ++r)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) sm[own + r * kSegWords + kNxt + i * 32] = g[r][i];
+  if (k == k_last || k == mom_prev) {
+#pragma unroll
+    for (int r = 0; r < S; ++r)
+      if ((si[r].fluid >> lane) & 1u) write_moments(si[r], lane, k == k_last, dr[r], ux[r], uy[r]);
   }
 }
 
-// The resident solve: n_steps time steps of the whole set.  words: step-buffer
-// size (storage elements) from the plan; halo: [2][halo_cap][9][32] tagged
-// words; tags epoch0 + 1 .. epoch0 + n_steps - 1 are published by this
-// launch.  Moments go to drho/ux/uy at the last step and to
-// drho/ux_prev/uy_prev at step mom_prev (-1: none).  tag_skew is 0, or 1
-// under the bounded-wait test hook (every wait then runs out).
-template <class T>
-__global__ void __launch_bounds__(kResidentMaxWarps * 32, 1)
+// The resident solve: n_steps (even) time steps of the whole set.  halo:
+// [2][halo_cap][3][32] published words; tags epoch0 + 1 .. epoch0 + n_steps - 1
+// are published by this launch.  Moments go to drho/ux/uy at the last step
+// and to drho/ux_prev/uy_prev at step mom_prev (-1: none).  tag_skew is 0, or
+// 1 under the bounded-wait test hook (every wait then runs out).
+// S: segments per warp, 1 or 2.
+template <class T, int FEAT, int S>
+__global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
     k_stream_collide_resident(const LatticeView* __restrict__ views, const SegRef* __restrict__ segs,
                               const int* __restrict__ n_segs, const int* __restrict__ seg_word_off,
-                              const int* __restrict__ seg_flags, const int* __restrict__ seg_offs, int words,
-                              unsigned long long* __restrict__ halo, int halo_cap, unsigned epoch0, int n_steps,
-                              int mom_prev, int* __restrict__ error, unsigned tag_skew) {
-  extern __shared__ __align__(16) unsigned char rsm[];
-  __shared__ OwnInfo oi;
-  __shared__ int s_order[kResidentMaxOwn], s_slot[kResidentMaxOwn];
-  __shared__ float2 s_rw[kResidentMaxOwn];  // (rho0, omega) of each slot's lattice
+                              const int* __restrict__ seg_flags, const int* __restrict__ seg_offs,
+                              HaloWord* __restrict__ halo, int halo_cap, unsigned epoch0, int n_steps, int mom_prev,
+                              int* __restrict__ error, unsigned tag_skew) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int s_nbq[Layout<S>::kSlots][8];  // list index of each neighbouring segment, or -1
+  __shared__ int s_order[Layout<S>::kSlots], s_slot[Layout<S>::kSlots];
+  __shared__ SlotInfo s_slots[Layout<S>::kSlots];
+  __shared__ PairInfo s_pairs[Layout<S>::kWarps];
   using P = Pop<T>;
+  constexpr int kBufWords = Layout<S>::kWords, kZeroWord = Layout<S>::kZero, kGhost0 = Layout<S>::kGhost0;
   const int nseg = n_segs[0];
-  const int G = gridDim.x;
   int s0, s1;
-  block_range(nseg, G, blockIdx.x, s0, s1);
-  const int n_own = s1 - s0;  // <= kResidentMaxOwn (checked by the plan)
-  const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // two step buffers, each a multiple of 16 bytes long (so that buffer 1,
-  // and the int scratch the prologue keeps in it, start 16-byte aligned),
-  // then the ghost-row table
-  const int stride = resident_buffer_stride(words);
-  T* buf0 = reinterpret_cast<T*>(rsm);
-  T* buf1 = buf0 + stride;
-  int* gp = reinterpret_cast<int*>(rsm + 2 * (size_t)stride * sizeof(T));
-  const int zero = words - 1;  // a word that stays 0 in both buffers
-  const int ghost0 = n_own * kSegWords;
+  block_range(nseg, gridDim.x, blockIdx.x, s0, s1);
+  const int n_own = s1 - s0;  // at most S per warp: the host sizes the grid by a bound on nseg
+  if (n_own > S * (int)(blockDim.x >> 5)) {
+    if (threadIdx.x == 0) atomicExch(error, 1);
+    return;
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* buf0 = sm;
 
-  // ---- once per launch: ranges, slots, ghost rows, source offsets ----
-  describe_range(views, segs, seg_word_off, seg_flags, seg_offs, s0, s1, oi);
+  // ---- once per launch: neighbours, slots, source addresses ----
+  for (int i = threadIdx.x; i < 8 * n_own; i += blockDim.x) {
+    const SegRef sr = segs[s0 + (i >> 3)];
+    const int p = i & 7;
+    s_nbq[i >> 3][p] = list_index(views, seg_word_off, seg_flags, seg_offs, sr.lattice,
+                                  (sr.yw >> kSegWordBits) + pos_dy(p),
+                                  (sr.yw & ((1 << kSegWordBits) - 1)) + pos_dw(p));
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {  // slots: published segments first
-    int j = 0;
-    for (int pass = 0; pass < 2; ++pass)
-      for (int t = 0; t < n_own; ++t)
-        if ((oi.pub[t] != 0) == (pass == 0)) {
-          s_order[j] = t;
-          s_slot[t] = j;
-          ++j;
-        }
+  if (warp == 0) {
+    // Slots.  A port cell's rules take as long as a collision, so segments with
+    // port cells go to slots of different warps, each beside one without.  The
+    // others follow with those that read other blocks first, so that they share
+    // warps and the remaining warps compute while these wait for their words.
+    unsigned port[2], touch[2], plain[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int t = lane + 32 * h;
+      bool remote = false, has_port = false;
+      if (t < n_own) {
+        for (int p = 0; p < 8; ++p) remote |= s_nbq[t][p] >= 0 && (s_nbq[t][p] < s0 || s_nbq[t][p] >= s1);
+        const SegRef sr = segs[s0 + t];
+        const LatticeView& L = views[sr.lattice];
+        const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
+        const uint32_t fl = ~L.mask[(long long)y * mask_stride(L.wpr) + w];
+        has_port = (w == 0 && (fl & 1u)) || (w == (L.nx - 1) >> 5 && ((fl >> ((L.nx - 1) & 31)) & 1u));
+      }
+      port[h] = __ballot_sync(kFull, has_port);
+      touch[h] = __ballot_sync(kFull, t < n_own && remote && !has_port);
+      plain[h] = __ballot_sync(kFull, t < n_own && !remote && !has_port);
+    }
+    const int n_port = __popc(port[0]) + __popc(port[1]), n_touch = __popc(touch[0]) + __popc(touch[1]);
+    const int m = min(n_port, n_own - n_port);  // pairs of a port and another segment
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int t = lane + 32 * h;
+      if (t >= n_own) continue;
+      auto rank = [&](const unsigned (&b)[2]) {
+        const unsigned below = (1u << lane) - 1u;
+        return h ? __popc(b[0]) + __popc(b[1] & below) : __popc(b[0] & below);
+      };
+      const bool is_port = (port[h] >> lane) & 1u;
+      const int i = is_port ? rank(port) : ((touch[h] >> lane) & 1u) ? rank(touch) : n_touch + rank(plain);
+      const int j = S == 1 ? (is_port ? i : n_port + i) : i < m ? 2 * i + (is_port ? 0 : 1) : m + i;
+      s_order[j] = t;
+      s_slot[t] = j;
+    }
   }
-  // ghost rows, each once (scratch in step buffer 1, unused until step 0 ends)
-  int* raw = reinterpret_cast<int*>(buf1);
-  const int npairs = collect_ghosts(oi, n_own, raw, raw + 12 * n_own, gp);
-  __syncthreads();  // the scratch is overwritten below
-  if (threadIdx.x < 32) {
-    P::st(buf0 + zero, 0.0f);
-    P::st(buf1 + zero, 0.0f);
-  }
+  if (threadIdx.x < 2) sm[threadIdx.x * kBufWords + kZeroWord] = 0.0f;
+  __syncthreads();
 
   const uint16_t* __restrict__ nbs = segment_flags(segs, n_segs);
-  // per slot r (j = warp + r W): source offsets of directions 1..8, packed
-  // 16-bit; the cell's offset in its lattice; flags; inlet speed
-  uint32_t offw[2][4];
-  int cell[2], lat[2], qj[2];
-  unsigned bits[2];  // bit 0 fluid, 1 inlet, 2 outlet, 3 zero-gradient outlet rule,
-                     // 4 constant-density outlet rule, 5 Zou-He ports; bits 8.. publish mask
-  float uin[2];
+  unsigned off[8];  // source words of directions 1..8 (two slots: 2w in the low half, 2w + 1 in the high)
+  const unsigned own = (unsigned)(S * warp * kSegWords + lane);
+  PairInfo& pi = s_pairs[warp];
+  unsigned flags = 0;
+  if (lane < 4) pi.vert[lane] = -1;
+  if (lane < 16) pi.edge[lane] = -1;
+  __syncwarp();
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int j = warp + r * W;
-    offw[r][0] = offw[r][1] = offw[r][2] = offw[r][3] = 0;
-    cell[r] = 0;
-    lat[r] = 0;
-    qj[r] = 0;
-    bits[r] = 0;
-    uin[r] = 0.0f;
-    if (j >= n_own) continue;
-    const int t = s_order[j];
-    const int q = s0 + t;
+  for (int r = 0; r < S; ++r) {
+    const int j = S * warp + r;
+    unsigned sf = 0;
+    if (j >= n_own) {  // an empty slot relaxes a resting cell into rows nobody reads
+      if (lane == 0) {
+        pi.rho0[r] = 1.0f;
+        pi.omega[r] = 1.0f;
+        pi.unit0[r] = 0;
+        s_slots[j] = SlotInfo{-1, -1, 0.0f, 0, 0, views, 0u};
+      }
+#pragma unroll
+      for (int i = 0; i < 9; ++i) buf0[j * kSegWords + i * 32 + lane] = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) off[i] = r ? off[i] | (unsigned)kZeroWord << 16 : (unsigned)kZeroWord;
+      continue;
+    }
+    const int t = s_order[j], q = s0 + t;
     const SegRef sr = segs[q];
     const LatticeView& L = views[sr.lattice];
     const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
@@ -332,238 +457,185 @@ __global__ void __launch_bounds__(kResidentMaxWarps * 32, 1)
     const bool fluid = !((mc >> lane) & 1u);
     const bool inlet = x == 0, outlet = x == L.nx - 1;
     const unsigned nb = nbs[(long long)q * 32 + lane];
-    const int base = j * kSegWords;
+    const bool plane = (FEAT & kFeatMirror) && L.mirror && y == 0;  // the row next to the symmetry plane
+    const int base = j * kSegWords, gbase = kGhost0 + j * kGhostWords;
 #pragma unroll
     for (int i = 1; i <= 8; ++i) {
-      int off = zero;
-      const int cx = cx_of(i), cy = cy_of(i);
+      int o = kZeroWord;
+      const int cx = cx_of(i);
       const bool unknown = (inlet && cx > 0) || (outlet && cx < 0);
       if (fluid && !unknown) {
         if ((nb >> (opp_of(i) - 1)) & 1u) {  // the source cell is solid: bounce-back
-          off = base + opp_of(i) * 32 + lane;
+          o = base + opp_of(i) * 32 + lane;
         } else {
-          const int sl = lane - cx, dy = -cy;
+          // next to the plane a diagonal from below is what the row-0 neighbour sent
+          // across it: NE from the west neighbour's SE, NW from the east one's SW
+          const bool image = plane && (i == 5 || i == 6);
+          const int si = image ? (i == 5 ? 8 : 7) : i;
+          const int sl = lane - cx, dy = image ? 0 : -cy_of(i);
           const int dw = sl < 0 ? -1 : sl > 31 ? 1 : 0;
-          const int slane = sl & 31;
           if (dy == 0 && dw == 0) {
-            off = base + i * 32 + slane;
+            o = base + si * 32 + sl;
           } else {
-            const int p = pos_of(dy, dw);
-            const int nq = oi.nbq[t][p];
-            if (nq >= s0 && nq < s1) {
-              off = s_slot[nq - s0] * kSegWords + i * 32 + slane;
-            } else if (nq >= 0) {
-              const int g = find_ghost(gp, npairs, (nq << 4) | i);
-              if (g >= 0) off = ghost0 + g * 32 + slane;
-            }  // nq < 0 cannot happen for a fluid source; the zero word keeps it harmless
+            const int nq = s_nbq[t][pos_of(dy, dw)];
+            if (nq >= s0 && nq < s1)
+              o = s_slot[nq - s0] * kSegWords + si * 32 + (sl & 31);
+            else if (nq >= 0)
+              o = gbase + ((cy_of(i) == 0) ? (i == 1 ? kGhostWest : kGhostEast) : ghost_row(i) * kGhostRow + 1 + sl);
+            // nq < 0 cannot happen for a fluid source; the zero word keeps it harmless
           }
         }
       }
-      offw[r][(i - 1) >> 1] |= (uint32_t)off << (16 * ((i - 1) & 1));
+      off[i - 1] = r ? off[i - 1] | (unsigned)o << 16 : (unsigned)o;
     }
-    cell[r] = y * L.pitch + x;
-    lat[r] = sr.lattice;
-    qj[r] = q;
-    bits[r] = (fluid ? 1u : 0u) | (inlet ? 2u : 0u) | (outlet ? 4u : 0u) |
-              (L.outlet_rule == LBM_OUT_NEUMANN ? 8u : 0u) | (L.outlet_rule == LBM_OUT_CONST_RHO ? 16u : 0u) |
-              (L.port_scheme == LBM_PORTS_ZOU_HE ? 32u : 0u) | (oi.pub[t] << 8);
-    uin[r] = inlet ? L.u_in[y] : 0.0f;
-    if (lane == 0) s_rw[j] = make_float2(L.rho0, L.omega);
-    // own populations from the canonical layout into step buffer 0
-    const T* F = static_cast<const T*>(L.f);
-    const int pl = (int)L.plane;
+    // what other blocks read of this segment, and what it reads of theirs
+    bool rem[8];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = F[i * pl + cell[r]];
-  }
-  __syncthreads();  // every source offset is known: the keys below may be replaced
-  // ghost rows of step 0 from the canonical layout; each key becomes the
-  // row's element offset in a halo parity, (segment * 9 + direction) * 32
-  for (int g = warp; g < npairs; g += W) {
-    const int e = gp[g];
-    const SegRef sr = segs[e >> 4];
-    const LatticeView& L = views[sr.lattice];
-    const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
+    for (int p = 0; p < 8; ++p) rem[p] = s_nbq[t][p] >= 0 && (s_nbq[t][p] < s0 || s_nbq[t][p] >= s1);
+    const bool side = rem[0] || rem[2];
+    if (rem[1] || rem[4] || rem[5]) sf |= kPubUp;
+    if (rem[3] || rem[6] || rem[7] || (plane && side)) sf |= kPubDown;
+    if (side) sf |= kPubSide;
+    auto word = [&](int p, int unit, int l, int value) {
+      return ((s_nbq[t][p] * 3 + unit) * kUnitWords + l) << 2 | value;
+    };
+    if (lane == 0) {
+      if (rem[1]) pi.vert[2 * r] = (s_nbq[t][1] * 3 + kUnitDown) * kUnitWords;
+      if (rem[3]) pi.vert[2 * r + 1] = (s_nbq[t][3] * 3 + kUnitUp) * kUnitWords;
+      if (rem[2]) pi.edge[8 * r + 0] = word(2, kUnitSide, 31, 0);
+      if (rem[0]) pi.edge[8 * r + 1] = word(0, kUnitSide, 0, 1);
+      if (rem[5]) pi.edge[8 * r + 2] = word(5, kUnitDown, 31, 2);
+      if (rem[4]) pi.edge[8 * r + 3] = word(4, kUnitDown, 0, 1);
+      if (rem[6]) pi.edge[8 * r + 4] = word(6, kUnitUp, 31, 1);
+      if (rem[7]) pi.edge[8 * r + 5] = word(7, kUnitUp, 0, 2);
+      if (plane && rem[2]) pi.edge[8 * r + 4] = word(2, kUnitDown, 31, 2);
+      if (plane && rem[0]) pi.edge[8 * r + 5] = word(0, kUnitDown, 0, 1);
+      pi.rho0[r] = L.rho0;
+      pi.omega[r] = L.omega;
+      pi.unit0[r] = q * 3 * kUnitWords;
+      const int ol = L.nx - 1 - (w << 5);
+      s_slots[j] = SlotInfo{w == 0 && !(mc & 1u) ? 0 : -1, ol < 32 && !((mc >> (ol & 31)) & 1u) ? ol : -1,
+                            w == 0 ? L.u_in[y] : 0.0f, L.port_scheme == LBM_PORTS_ZOU_HE,
+                            (long long)y * L.pitch + (w << 5), &L, ~mc};
+    }
+    if (__any_sync(kFull, fluid && (inlet || outlet))) sf |= kHasPort;
+    if (L.outlet_rule == LBM_OUT_NEUMANN) sf |= kNeumann;
+    if ((FEAT & kFeatModels) && L.collision != LBM_COLLIDE_BGK) sf |= kSlotModel;
+    flags |= sf << (16 * r);
+    // own populations and the ghost words of step 0 from the canonical layout
     const T* F = static_cast<const T*>(L.f);
-    buf0[ghost0 + g * 32 + lane] = F[(e & 15) * (int)L.plane + y * L.pitch + (w << 5) + lane];
-    __syncwarp();
-    if (lane == 0) gp[g] = ((e >> 4) * 9 + (e & 15)) * 32;
+    const int pl = (int)L.plane, cell = y * L.pitch + x;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = P::ld(F + i * pl + cell);
+    float* gw = buf0 + gbase;
+    if (rem[1]) {
+      gw[1 + lane] = P::ld(F + 4 * pl + cell + L.pitch);
+      gw[kGhostRow + 1 + lane] = P::ld(F + 7 * pl + cell + L.pitch);
+      gw[2 * kGhostRow + 1 + lane] = P::ld(F + 8 * pl + cell + L.pitch);
+    }
+    if (rem[3]) {
+      gw[3 * kGhostRow + 1 + lane] = P::ld(F + 2 * pl + cell - L.pitch);
+      gw[4 * kGhostRow + 1 + lane] = P::ld(F + 5 * pl + cell - L.pitch);
+      gw[5 * kGhostRow + 1 + lane] = P::ld(F + 6 * pl + cell - L.pitch);
+    }
+    if (lane == 0) {
+      if (rem[2]) gw[kGhostWest] = P::ld(F + 1 * pl + cell - 1);
+      if (rem[5]) gw[2 * kGhostRow] = P::ld(F + 8 * pl + cell + L.pitch - 1);
+      if (rem[6]) gw[4 * kGhostRow] = P::ld(F + 5 * pl + cell - L.pitch - 1);
+      if (plane && rem[2]) gw[4 * kGhostRow] = P::ld(F + 8 * pl + cell - 1);
+    }
+    if (lane == 31) {
+      if (rem[0]) gw[kGhostEast] = P::ld(F + 3 * pl + cell + 1);
+      if (rem[4]) gw[kGhostRow + 33] = P::ld(F + 7 * pl + cell + L.pitch + 1);
+      if (rem[7]) gw[5 * kGhostRow + 33] = P::ld(F + 6 * pl + cell - L.pitch + 1);
+      if (plane && rem[0]) gw[5 * kGhostRow + 33] = P::ld(F + 7 * pl + cell + 1);
+    }
   }
+  const SlotInfo* si = s_slots + S * warp;
+  if (lane == 0) pi.flags = flags;
+  // ghost words are read exactly by the segments that publish
+  const bool ghosts = (flags & (kPublishes << 16 | kPublishes)) != 0;
 
-  // ---- the time steps ----
-  for (int k = 0; k < n_steps; ++k) {
-    T* cur = (k & 1) ? buf1 : buf0;
-    T* nxt = (k & 1) ? buf0 : buf1;
-    int failed = 0;
-    if (k > 0) {  // ghost rows of step k: the words of step k - 1, tag epoch0 + k
-      const unsigned want = epoch0 + (unsigned)k + tag_skew;
-      const unsigned long long* hb = halo + (size_t)((k - 1) & 1) * halo_cap * kSegWords;
-      // a warp's rows are g = warp + u W: up to kFetch of them in flight at once
-      for (int g0 = warp; g0 < npairs && !failed; g0 += kFetch * W) {
-        unsigned long long v[kFetch];
-#pragma unroll
-        for (int u = 0; u < kFetch; ++u) {
-          const int g = g0 + u * W;
-          v[u] = g < npairs ? ld_relaxed_u64(hb + gp[g] + lane) : (unsigned long long)want << 32;
-        }
-        unsigned spins = 0;
-        for (;;) {
-          bool ready = true;
-#pragma unroll
-          for (int u = 0; u < kFetch; ++u) ready &= (unsigned)(v[u] >> 32) == want;
-          if (__all_sync(kFull, ready)) break;
-#pragma unroll
-          for (int u = 0; u < kFetch; ++u) {
-            const int g = g0 + u * W;
-            if (g < npairs && (unsigned)(v[u] >> 32) != want) v[u] = ld_relaxed_u64(hb + gp[g] + lane);
-          }
-          ++spins;
-          if (spins > kResidentSpinLimit ||
-              ((spins & 255u) == 0 && __any_sync(kFull, ld_relaxed_s32(error) != 0))) {
-            failed = 1;
-            break;
-          }
-        }
-        if (failed) break;
-#pragma unroll
-        for (int u = 0; u < kFetch; ++u) {
-          const int g = g0 + u * W;
-          if (g < npairs) P::st(cur + ghost0 + g * 32 + lane, __uint_as_float((unsigned)v[u]));
-        }
-      }
-    }
-    if (__syncthreads_or(failed)) {
-      if (threadIdx.x == 0) atomicExch(error, 1);
-      return;  // the global layout keeps the state from before the launch
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int j = warp + r * W;
-      if (j >= n_own) break;
-      const int base = j * kSegWords;
-      float g[9];
-      g[0] = P::ld(cur + base + lane);
-#pragma unroll
-      for (int i = 1; i <= 8; ++i) g[i] = P::ld(cur + ((offw[r][(i - 1) >> 1] >> (16 * ((i - 1) & 1))) & 0xffffu));
-      const bool fluid = bits[r] & 1u, inlet = bits[r] & 2u, outlet = bits[r] & 4u;
-      if (bits[r] & 8u) {  // zero-gradient outlet: cell nx-2 is the lane to the left
-        const float n3 = __shfl_up_sync(kFull, g[3], 1);
-        const float n6 = __shfl_up_sync(kFull, g[6], 1);
-        const float n7 = __shfl_up_sync(kFull, g[7], 1);
-        if (outlet) {
-          g[3] = n3;
-          g[6] = n6;
-          g[7] = n7;
-        }
-      }
-      if (fluid) {
-        const float2 rw = s_rw[j];
-        const float rho0 = rw.x;
-        const int scheme = (bits[r] & 32u) ? LBM_PORTS_ZOU_HE : LBM_PORTS_REGULARIZED;
-        if (inlet) {
-          inlet_rule(g, uin[r], rho0, scheme);
-        } else if (outlet && (bits[r] & 16u)) {
-          outlet_rule(g, rho0, scheme);
-        }
-        float drho, ux, uy;
-        bgk(g, rho0, rw.y, drho, ux, uy);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) P::st(nxt + base + i * 32 + lane, g[i]);
-        if (k == n_steps - 1) {
-          const LatticeView& L = views[lat[r]];
-          L.drho[cell[r]] = drho;
-          L.ux[cell[r]] = ux;
-          L.uy[cell[r]] = uy;
-        } else if (k == mom_prev) {
-          const LatticeView& L = views[lat[r]];
-          L.drho[cell[r]] = drho;
-          L.ux_prev[cell[r]] = ux;
-          L.uy_prev[cell[r]] = uy;
-        }
-      }
-      const unsigned pub = bits[r] >> 8;
-      if (pub && k + 1 < n_steps) {
-        unsigned long long* hd = halo + ((size_t)(k & 1) * halo_cap + qj[r]) * kSegWords + lane;
-        const unsigned long long tag = (unsigned long long)(epoch0 + (unsigned)k + 1u) << 32;
-#pragma unroll
-        for (int i = 1; i <= 8; ++i)
-          if ((pub >> i) & 1u)
-            st_relaxed_u64(hd + i * 32, tag | __float_as_uint(fluid ? round_to_storage<T>(g[i]) : 0.0f));
-      }
-    }
+  // ---- the time steps, two per turn: step k reads buffer k & 1 ----
+  // A warp whose words do not come sets the error word, which ends every other
+  // wait, and idles to the next common check; the block leaves there.
+  const int parity = halo_cap * 3 * kUnitWords;
+  int failed = 0;
+  auto turn = [&](int k) {
+    if ((k & 127) == 0) return __syncthreads_or(failed) == 0;
+    __syncthreads();
+    return true;
+  };
+  for (int k = 0; k < n_steps; k += 2) {
+    if (!turn(k)) break;
+    if (k > 0 && ghosts && !failed)
+      failed = !fetch_ghosts<S>(sm, pi, halo, parity, epoch0 + (unsigned)k + tag_skew, lane, error);
+    if (!failed) warp_step<T, FEAT, S, 0>(sm, off, own, k, n_steps - 1, mom_prev, epoch0, pi, si, halo, 0, lane);
+    __syncthreads();
+    if (ghosts && !failed)
+      failed = !fetch_ghosts<S>(sm + kBufWords, pi, halo, 0, epoch0 + (unsigned)k + 1u + tag_skew, lane, error);
+    if (!failed) warp_step<T, FEAT, S, 1>(sm, off, own, k + 1, n_steps - 1, mom_prev, epoch0, pi, si, halo, parity, lane);
   }
-  // ---- the final state back to the canonical layout ----
-  const T* fin = (n_steps & 1) ? buf1 : buf0;
+  if (__syncthreads_or(failed)) return;  // the global layout keeps the state from before the launch
+  // ---- the final state (buffer 0: an even number of steps) to the canonical layout ----
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int j = warp + r * W;
-    if (j >= n_own || !(bits[r] & 1u)) continue;
-    const LatticeView& L = views[lat[r]];
-    T* F = static_cast<T*>(L.f);
+  for (int r = 0; r < S; ++r) {
+    if (!((si[r].fluid >> lane) & 1u)) continue;
+    const LatticeView& L = *si[r].L;
+    T* F = static_cast<T*>(L.f) + si[r].row + lane;
     const int pl = (int)L.plane;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) F[i * pl + cell[r]] = fin[j * kSegWords + i * 32 + lane];
+    for (int i = 0; i < 9; ++i) P::st(F + i * pl, sm[own + r * kSegWords + i * 32]);
+  }
+}
+
+template <class T, int S>
+void* resident_kernel(int features) {
+  switch (features) {
+    case 0: return (void*)k_stream_collide_resident<T, 0, S>;
+    case kFeatModels: return (void*)k_stream_collide_resident<T, kFeatModels, S>;
+    case kFeatMirror: return (void*)k_stream_collide_resident<T, kFeatMirror, S>;
+    case kFeatModels | kFeatMirror: return (void*)k_stream_collide_resident<T, kFeatModels | kFeatMirror, S>;
+    default: return nullptr;
   }
 }
 
 template <class T>
-void* resident_kernel() {
-  return (void*)k_stream_collide_resident<T>;
+void* resident_kernel(int features, int per_warp) {
+  return per_warp == 1 ? resident_kernel<T, 1>(features) : resident_kernel<T, 2>(features);
 }
 
-void* resident_kernel_for(int precision) {
+void* resident_kernel_for(int precision, int features, int per_warp) {
   switch (precision) {
-    case LBM_F32: return resident_kernel<float>();
-    case LBM_BF16_SHIFTED: return resident_kernel<__nv_bfloat16>();
-    case LBM_F16_SHIFTED: return resident_kernel<__half>();
+    case LBM_F32: return resident_kernel<float>(features, per_warp);
+    case LBM_BF16_SHIFTED: return resident_kernel<__nv_bfloat16>(features, per_warp);
+    case LBM_F16_SHIFTED: return resident_kernel<__half>(features, per_warp);
     default: return nullptr;
   }
 }
 
 }  // namespace
 
-size_t resident_smem_bytes(int precision, int words, int pairs) {
-  const size_t sb = precision == LBM_F32 ? 4 : 2;
-  return 2 * (size_t)resident_buffer_stride(words) * sb + (size_t)(pairs > 0 ? pairs : 1) * sizeof(int);
-}
+size_t resident_halo_bytes(int segments) { return (size_t)2 * segments * 3 * kUnitWords * sizeof(HaloWord); }
 
-int resident_max_smem() {
-  int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-    return 0;
-  // the kernel's static shared memory (the block's segment table) comes on top
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, resident_kernel_for(LBM_F32)) != cudaSuccess) return 0;
-  return v - (int)fa.sharedSizeBytes;
-}
-
-cudaError_t launch_resident_plan(const LatticeView* views, const SegRef* segs, const int* n_segs,
-                                 const int* seg_word_off, const int* seg_flags, const int* seg_offs, int sm_count,
-                                 int* out, cudaStream_t stream) {
-  cudaError_t e = cudaMemsetAsync(out, 0, 4 * sizeof(int), stream);
-  if (e != cudaSuccess) return e;
-  k_resident_plan<<<sm_count, 64, 0, stream>>>(views, segs, n_segs, seg_word_off, seg_flags, seg_offs, sm_count, out);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stream_collide_resident(int precision, const LatticeView* views, const SegRef* segs,
+cudaError_t launch_stream_collide_resident(int precision, int features, const LatticeView* views, const SegRef* segs,
                                            const int* n_segs, const int* seg_word_off, const int* seg_flags,
-                                           const int* seg_offs, const ResidentShape& rs,
-                                           unsigned long long* halo, int halo_cap, unsigned epoch0, int n_steps,
-                                           int mom_prev, int* error, cudaStream_t stream) {
-  void* k = resident_kernel_for(precision);
+                                           const int* seg_offs, const ResidentShape& rs, void* halo, int halo_cap,
+                                           unsigned epoch0, int n_steps, int mom_prev, int* error,
+                                           cudaStream_t stream) {
+  void* k = resident_kernel_for(precision, features, rs.per_warp);
   // under the test hook every wait expects a tag that nobody writes
   unsigned tag_skew = barrier_timeout_test() ? 1u : 0u;
-  if (!k || rs.grid < 1 || rs.warps < 1 || rs.warps > kResidentMaxWarps || rs.words < kSegWords + 1 ||
-      rs.words > 65536 || n_steps < 1 || halo_cap < 1)
+  if (!k || rs.grid < 1 || rs.warps < 1 ||
+      rs.warps > (rs.per_warp == 1 ? kResidentMaxWarps : kResidentMaxOwn / 2) || n_steps < 2 || (n_steps & 1) ||
+      halo_cap < 1)
     return cudaErrorInvalidValue;
-  const size_t smem = resident_smem_bytes(precision, rs.words, rs.pairs);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int smem = 2 * (int)sizeof(float) * (rs.per_warp == 1 ? Layout<1>::kWords : Layout<2>::kWords);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&views, (void*)&segs, (void*)&n_segs, (void*)&seg_word_off, (void*)&seg_flags,
-                  (void*)&seg_offs, (void*)&rs.words, (void*)&halo, (void*)&halo_cap, (void*)&epoch0,
-                  (void*)&n_steps, (void*)&mom_prev, (void*)&error, (void*)&tag_skew};
+                  (void*)&seg_offs, (void*)&halo, (void*)&halo_cap, (void*)&epoch0, (void*)&n_steps,
+                  (void*)&mom_prev, (void*)&error, (void*)&tag_skew};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;  // every block resident: neighbours' words always come
   attr[0].val.cooperative = 1;
