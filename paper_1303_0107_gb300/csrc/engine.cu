@@ -309,13 +309,6 @@ lbm_status reserve_oc(Engine* E, const SetLayout& X) {
   return LBM_OK;
 }
 
-// The list's length, read after the stream has been synchronised.
-void take_seg_count(Engine* E) {
-  if (!E->nseg_copied) return;
-  E->nseg_copied = false;
-  E->seg_bound = *E->h_nseg;
-}
-
 lbm_status launch_pair(Engine* E, int moments) {
   // moments: 0 none, 1 into drho/ux/uy, 2 into drho/ux_prev/uy_prev
   const LatticeView* views = static_cast<const LatticeView*>(E->L.views.p);
@@ -1096,9 +1089,15 @@ lbm_status ensure_pairs(Engine* E) {
   return LBM_OK;
 }
 
+void take_seg_count(Engine* E) {
+  if (!E->nseg_copied) return;
+  E->nseg_copied = false;
+  E->seg_bound = *E->h_nseg;
+}
+
 lbm_status resident_prepare(Engine* E, bool* ok) {
   *ok = false;
-  if (E->fixed_grid || E->n() == 0 || debug_sync()) return LBM_OK;
+  if (E->n() == 0 || debug_sync()) return LBM_OK;
   if (E->nseg_copied && E->seg_bound > (long long)kResidentMaxOwn * E->sm_count) {  // the bound is too wide: count
     CU(cudaStreamSynchronize(E->stream));
     take_seg_count(E);
@@ -1401,6 +1400,11 @@ lbm_status choose_resident(Engine* E, int64_t n_steps) {
       n_steps < kResidentMinSteps)
     return LBM_OK;
   lbm_status st = resident_prepare(E, &E->resident_now);
+  if (st == LBM_ERR_OOM) {  // no room for the halo words: the per-phase kernels need none
+    cudaGetLastError();
+    E->resident_now = false;
+    st = LBM_OK;
+  }
   E->resident_by_rule = E->resident_now;
   return st;
 }

@@ -178,6 +178,11 @@ lbm_status rebuild_worklist(Engine* E);
 // Shape and halo buffer of a resident launch over the current work-list;
 // *ok: the set fits the chip.
 lbm_status resident_prepare(Engine* E, bool* ok);
+// Whether the next n_steps of E step on the chip by rule (E->resident_now).
+lbm_status choose_resident(Engine* E, int64_t n_steps);
+// Take the work-list's length copied by the last rebuild (the stream has been
+// synchronised since).
+void take_seg_count(Engine* E);
 // Compacted fluid-cell tasks: whether the set may use them (plain BGK, no
 // zero-gradient outlet), and the list built for the current work-list.
 bool cells_eligible(const Engine* E);

@@ -79,7 +79,7 @@ size_t engine_buffer_bytes(const Engine* E) {
   size_t b = 0;
   for (const GrowBuf* g : {&E->L.views, &E->L.word_off, &E->L.seg_word_off, &E->XL.views, &E->XL.word_off,
                            &E->XL.seg_word_off, &E->segs, &E->n_segs, &E->seg_scratch, &E->partials, &E->result,
-                           &E->fluid_dev, &E->n_swap_dev, &E->dense_f, &E->oc_buf, &E->bar})
+                           &E->fluid_dev, &E->n_swap_dev, &E->dense_f, &E->oc_buf, &E->bar, &E->halo})
     b += g->cap;
   return b;
 }
@@ -270,11 +270,17 @@ void lbm_server_s::loop() {
     if (!which.empty()) s = enqueue_exchange(E, which, n_swap.data());
     int64_t S = cfg.max_tick_steps;
     for (const Slot& x : slots) S = std::min(S, x.steps_left);
+    // a set that fits the chip steps there (one to three requests most of the
+    // time at light load)
+    if (s == LBM_OK) s = choose_resident(E, S);
     if (s == LBM_OK) s = enqueue_steps_and_reduce(E, S, false);
     if (s == LBM_OK && cudaStreamSynchronize(E->stream) != cudaSuccess)
       s = fail(LBM_ERR_CUDA, "server tick");
+    if (s == LBM_OK && *E->h_bar_error != 0)
+      s = fail(LBM_ERR_TIMEOUT, "step kernel: a bounded device wait gave up");
+    take_seg_count(E);
     if (s != LBM_OK) {
-      fail_all(s == LBM_ERR_OOM ? LBM_ERR_OOM : LBM_ERR_CUDA);
+      fail_all(s == LBM_ERR_OOM || s == LBM_ERR_TIMEOUT ? s : LBM_ERR_CUDA);
       return;
     }
     std::vector<int32_t> status(n, LBM_OK);
