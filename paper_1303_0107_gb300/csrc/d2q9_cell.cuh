@@ -181,20 +181,17 @@ __device__ __forceinline__ void relax_pair2(F2& gi, F2& go, F2 cu, F2 w, F2 r3, 
   go = f2_fma(omega, f2_sub(eo, go), go);
 }
 
-__device__ __forceinline__ void bgk2(float (&a)[9], float (&b)[9], F2 rho0, F2 omega, float& dra, float& uxa,
-                                     float& uya, float& drb, float& uxb, float& uyb) {
-  F2 g[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) g[i] = f2(a[i], b[i]);
-  const F2 drho = f2_add(f2_add(f2_add(f2_add(g[0], g[1]), f2_add(g[2], g[3])),
-                                f2_add(f2_add(g[4], g[5]), f2_add(g[6], g[7]))), g[8]);
+__device__ __forceinline__ void bgk2(F2 (&g)[9], F2 rho0, F2 omega, F2& drho, F2& ux, F2& uy) {
+  drho = f2_add(f2_add(f2_add(f2_add(g[0], g[1]), f2_add(g[2], g[3])),
+                       f2_add(f2_add(g[4], g[5]), f2_add(g[6], g[7]))), g[8]);
   const F2 rho = f2_add(rho0, drho);
   const F2 jx = f2_add(f2_add(f2_sub(g[1], g[3]), f2_sub(g[5], g[7])), f2_sub(g[8], g[6]));
   const F2 jy = f2_add(f2_add(f2_sub(g[2], g[4]), f2_sub(g[5], g[7])), f2_sub(g[6], g[8]));
   float rl, rh;
   f2_split(rho, rl, rh);
   const F2 inv = f2(__frcp_rn(rl), __frcp_rn(rh));  // correctly rounded: the value of 1.0f / rho
-  const F2 ux = f2_mul(jx, inv), uy = f2_mul(jy, inv);
+  ux = f2_mul(jx, inv);
+  uy = f2_mul(jy, inv);
   const F2 t0 = f2_fma(f2_mul(f2_c(-1.5f), rho), f2_fma(ux, ux, f2_mul(uy, uy)), drho);
   const F2 r3 = f2_mul(f2_c(3.0f), rho), r3n = f2_mul(f2_c(-3.0f), rho), r45 = f2_mul(f2_c(4.5f), rho);
   relax_pair2(g[1], g[3], ux, f2_c(kW1), r3, r3n, r45, t0, omega);
@@ -205,6 +202,15 @@ __device__ __forceinline__ void bgk2(float (&a)[9], float (&b)[9], F2 rho0, F2 o
   g[2] = f2_sub(f2_add(jy, g[4]), f2_add(f2_sub(g[5], g[7]), f2_sub(g[6], g[8])));
   g[0] = f2_sub(drho, f2_add(f2_add(f2_add(g[1], g[2]), f2_add(g[3], g[4])),
                              f2_add(f2_add(g[5], g[6]), f2_add(g[7], g[8]))));
+}
+
+// The same on the two cells' arrays, the moments taken apart.
+__device__ __forceinline__ void bgk2(float (&a)[9], float (&b)[9], F2 rho0, F2 omega, float& dra, float& uxa,
+                                     float& uya, float& drb, float& uxb, float& uyb) {
+  F2 g[9], drho, ux, uy;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) g[i] = f2(a[i], b[i]);
+  bgk2(g, rho0, omega, drho, ux, uy);
 #pragma unroll
   for (int i = 0; i < 9; ++i) f2_split(g[i], a[i], b[i]);
   f2_split(drho, dra, drb);

@@ -445,7 +445,22 @@ StepConfig resident_config(const Engine* E) {
   return c;
 }
 
+// Two sweeps, there and back.
+lbm_status run_sweeps(Engine* E) {
+  const Member* m = E->m[0];
+  const SweepList sl = sweep_list(m->nx, m->ny, E->sweep_buf.p);
+  const LatticeView& L = E->L.h_views[0];
+  int* error = &static_cast<StepBarrier*>(E->bar.p)->error;
+  CU(launch_sweep(L, m->f, E->second.p, sl, kSweepBlocks * E->sm_count, error, E->stream));
+  CU(launch_sweep(L, E->second.p, m->f, sl, kSweepBlocks * E->sm_count, error, E->stream));
+  return LBM_OK;
+}
+
 lbm_status run_plain_pairs(Engine* E, int64_t pairs) {
+  for (; E->sweep_now && pairs >= kSweepSteps; pairs -= kSweepSteps) {
+    lbm_status st = run_sweeps(E);
+    if (st != LBM_OK) return st;
+  }
   if (E->step.persistent == 1 && !debug_sync()) return run_persistent(E, pairs);
   if (debug_sync()) {
     for (int64_t k = 0; k < pairs; ++k) {
@@ -979,7 +994,8 @@ Engine::~Engine() {
     for (Member* x : m) delete x;
   for (GrowBuf* b : {&L.views, &L.word_off, &L.seg_word_off, &XL.views, &XL.word_off, &XL.seg_word_off, &segs,
                      &n_segs, &seg_scratch, &partials, &result, &fluid_dev, &n_swap_dev, &dense_f, &oc_buf, &bar,
-                     &best, &halo, &cell_list, &cell_scan, &pair_list, &pair_scan})
+                     &best, &halo, &cell_list, &cell_scan, &pair_list, &pair_scan,
+                     &sweep_buf, &second})
     b->release();
   if (h_bar_error) cudaFreeHost(h_bar_error);
   if (h_result) cudaFreeHost(h_result);
@@ -1009,6 +1025,7 @@ lbm_status engine_new(int precision, int residual_every, void* cuda_stream, bool
   int dev = 0;
   CUE(cudaGetDevice(&dev));
   CUE(cudaDeviceGetAttribute(&E->sm_count, cudaDevAttrMultiProcessorCount, dev));
+  CUE(cudaDeviceGetAttribute(&E->l2_bytes, cudaDevAttrL2CacheSize, dev));
   if (cuda_stream) {
     E->stream = static_cast<cudaStream_t>(cuda_stream);
   } else {
@@ -1029,6 +1046,7 @@ lbm_status engine_new(int precision, int residual_every, void* cuda_stream, bool
 lbm_status rebuild_worklist(Engine* E) {
   E->cells_valid = false;
   E->pairs_valid = false;
+  E->sweep_valid = false;
   for (Engine* g : E->groups) {  // the groups' lists follow the members' masks
     lbm_status st = rebuild_worklist(g);
     if (st != LBM_OK) return st;
@@ -1354,7 +1372,7 @@ lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
 
 lbm_status enqueue_steps_and_reduce(Engine* E, int64_t n_steps, bool with_res) {
   lbm_status st;
-  E->bar_used = false;
+  E->bar_used = E->sweep_now;
   {
     NvtxRange nvtx("lbm_time_steps");
     CU(cudaEventRecord(E->ev_begin, E->stream));
@@ -1409,10 +1427,83 @@ lbm_status choose_resident(Engine* E, int64_t n_steps) {
   return st;
 }
 
+// LBM_SWEEP=0 in the environment keeps solves out of sweeps, LBM_SWEEP=1 takes
+// them whatever the size (tests).
+bool sweep_enabled(bool* forced) {
+  const char* e = std::getenv("LBM_SWEEP");
+  *forced = e && e[0] == '1';
+  return !(e && e[0] == '0');
+}
+
+// The rule: sweeps where DRAM bounds the per-phase kernels and the tiles are
+// filled well, that is where the populations of the fluid cells exceed the L2
+// cache and the tile rows cost at most a tenth of a cost unit per fluid cell
+// (a row of 120 open cells costs 8).  Measured on FP32, us per step, sweeps /
+// the per-phase kernel the tuning picks:
+//   fluid populations  cost per cell  lattice
+//          605 MB          0.07       8192 x 4096, 16 channels   114 / 193
+//          144 MB          0.07       4000 x 2000,  4 channels    35 /  47
+//           81 MB          0.08       3000 x 1500, 16 channels    24 /  20
+//           36 MB          0.07       2000 x 1000,  8 channels    13 / 8.4
+//           92 MB          0.2        tree in 8192 x 4096         50 /  34
+// (a tree's narrow vessels leave most of a tile's columns idle: beyond the L2
+// cache the per-phase kernels run at about 11.5 ps per cell and step, sweeps at
+// 0.1 ns per cost unit and step).  With 16-bit populations the per-phase
+// kernels move half the bytes and are as fast (120 us for the first lattice,
+// sweeps 125), so those keep to them.
+lbm_status choose_sweep(Engine* E, int64_t n_steps) {
+  E->sweep_now = false;
+  bool forced = false;
+  if (E->resident_now || E->precision != LBM_F32 || E->shape_fixed || E->n() != 1 || E->features != 0 ||
+      E->fixed_grid || E->in_group || E->m[0]->p.outlet == LBM_OUT_NEUMANN || n_steps < 4 * kSweepSteps ||
+      !sweep_enabled(&forced) || !autotune_enabled() || debug_sync())
+    return LBM_OK;
+  const Member* m = E->m[0];
+  const size_t cell_bytes = 9 * sizeof(float), bytes = cell_bytes * m->plane, rows = (size_t)sweep_rows(m->nx, m->ny);
+  if (!forced && bytes <= (size_t)E->l2_bytes) return LBM_OK;
+  if (m->ny >= 1 << kSweepRowBits || rows / m->ny > (size_t)1 << (31 - kSweepRowBits) || rows >= (size_t)1 << 26)
+    return LBM_OK;  // more than a list entry and the sums hold
+  if (!E->sweep_valid) {
+    cudaError_t e = E->sweep_buf.reserve(sweep_list(m->nx, m->ny, nullptr).ints * sizeof(int));
+    if (e == cudaErrorMemoryAllocation) {  // the per-phase kernels need none of this
+      cudaGetLastError();
+      return LBM_OK;
+    }
+    CU(e);
+    const SweepList list = sweep_list(m->nx, m->ny, E->sweep_buf.p);
+    CU(launch_build_sweep(E->L.h_views[0], list, E->stream));
+    int cost = 0;
+    unsigned long long fluid = 0;
+    CU(cudaMemcpyAsync(&cost, list.total_cost, sizeof(cost), cudaMemcpyDeviceToHost, E->stream));
+    CU(cudaMemcpyAsync(&fluid, E->fluid_dev.p, sizeof(fluid), cudaMemcpyDeviceToHost, E->stream));
+    CU(cudaStreamSynchronize(E->stream));
+    E->sweep_pays = fluid * cell_bytes > (size_t)E->l2_bytes && (unsigned long long)cost * 10 <= fluid;
+    E->sweep_valid = true;
+  }
+  if (!E->sweep_pays && !forced) return LBM_OK;
+  if (E->second.cap < bytes) {
+    // a second buffer only out of plenty: what else the program allocates fits as before
+    size_t free_bytes = 0, all = 0;
+    CU(cudaMemGetInfo(&free_bytes, &all));
+    if (bytes > free_bytes / 8) return LBM_OK;
+    cudaError_t e = E->second.reserve(bytes);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      return LBM_OK;
+    }
+    CU(e);
+  }
+  if (!E->tuned) E->step = pairs_shape(E, 4, kDefaultGridScale);  // the few steps around the sweeps
+  CU(cudaMemsetAsync(&static_cast<StepBarrier*>(E->bar.p)->error, 0, sizeof(int), E->stream));
+  E->sweep_now = true;
+  return LBM_OK;
+}
+
 lbm_status enqueue_solve(Engine* E, int64_t n_steps) {
   lbm_status cst = choose_resident(E, n_steps);
+  if (cst == LBM_OK) cst = choose_sweep(E, n_steps);
   if (cst != LBM_OK) return cst;
-  if (n_steps >= 256 && !E->resident_now) {
+  if (n_steps >= 256 && !E->resident_now && !E->sweep_now) {
     lbm_status st = ensure_groups(E);
     if (st != LBM_OK) return st;
   }
@@ -1422,7 +1513,7 @@ lbm_status enqueue_solve(Engine* E, int64_t n_steps) {
         lbm_status st = autotune(g);
         if (st != LBM_OK) return st;
       }
-  } else if (!E->tuned && n_steps >= 256 && !E->resident_now) {
+  } else if (!E->tuned && n_steps >= 256 && !E->resident_now && !E->sweep_now) {
     lbm_status st = autotune(E);
     if (st != LBM_OK) return st;
   }

@@ -99,7 +99,7 @@ struct Engine {
   bool own_stream = false;
   bool own_members = true;  // handles and batches own their members; the server does not
   bool fixed_grid = false;  // step grid sized for the device, not for the current list
-  int sm_count = 0;
+  int sm_count = 0, l2_bytes = 0;
   std::vector<Member*> m;
 
   SetLayout L;   // every member: time steps, reductions, work-list
@@ -139,6 +139,13 @@ struct Engine {
   // work-list is rebuilt
   GrowBuf pair_list, pair_scan;
   bool pairs_valid = false;
+
+  // sweeps (sweep.cu): the row list with its scan buffers, valid until the
+  // work-list is rebuilt, and the second population buffer
+  GrowBuf sweep_buf, second;
+  bool sweep_valid = false;
+  bool sweep_pays = false;  // the rule's answer for the list
+  bool sweep_now = false;   // the solve being enqueued steps in sweeps
 
   cudaGraphExec_t graphs[4] = {nullptr, nullptr, nullptr, nullptr};  // 512, 64, 8 and 1 pairs
   // views, segs (or the cell or paired list), n_segs, shape, cell prefix (or paired count), layout build
@@ -187,6 +194,8 @@ void take_seg_count(Engine* E);
 // zero-gradient outlet), and the list built for the current work-list.
 bool cells_eligible(const Engine* E);
 lbm_status ensure_cells(Engine* E);
+// Sweeps: whether the next n_steps of E run in them (E->sweep_now).
+lbm_status choose_sweep(Engine* E, int64_t n_steps);
 bool pairs_eligible(const Engine* E);
 lbm_status ensure_pairs(Engine* E);
 

@@ -236,6 +236,30 @@ cudaError_t launch_stream_collide_resident(int precision, int features, const La
                                            unsigned epoch0, int n_steps, int mom_prev, int* error,
                                            cudaStream_t stream);
 
+// ---- sweeps (sweep.cu) -------------------------------------------------------
+// kSweepSteps time steps of one plain FP32 BGK lattice (no zero-gradient
+// outlet) in one pass over memory, from population buffer F to buffer G (both
+// of the lattice's layout; G's solid cells are left alone).
+constexpr int kSweepSteps = 4;
+constexpr int kSweepBlocks = 2;    // blocks per SM
+constexpr int kSweepRowBits = 19;  // list entry: tile << 19 | row
+long long sweep_rows(int nx, int ny);  // rows of all tiles
+// The rows of all tiles that hold fluid, with their costs, and what builds
+// them, carved from one device buffer (a null buffer gives the size alone).
+struct SweepList {
+  int *flags, *offs, *work, *work_before, *tmp;
+  int *list, *cost;
+  void* states;
+  const int *n_rows, *total_cost;
+  size_t ints;  // of the buffer
+};
+SweepList sweep_list(int nx, int ny, void* buffer);
+cudaError_t launch_build_sweep(const LatticeView& L, const SweepList& s, cudaStream_t stream);
+// A programmatic dependent launch like launch_stream_collide; *error is set
+// when a copy did not arrive.
+cudaError_t launch_sweep(const LatticeView& L, const void* F, void* G, const SweepList& s, int grid, int* error,
+                         cudaStream_t stream);
+
 // ---- geometry / work-list (worklist.cu) ------------------------------------
 cudaError_t launch_pack_mask(const uint8_t* cells, int nx, int ny, int wpr, uint32_t* mask,
                              cudaStream_t stream);
