@@ -408,35 +408,40 @@ lbm_status run_persistent(Engine* E, int64_t pairs) {
 // that it lies in the last launch.
 constexpr int64_t kMaxResidentSteps = (int64_t)1 << 28;
 
+// The halo buffer and the error word: a member group uses its batch's.
+Engine* halo_engine(Engine* E) { return E->resident_parent ? E->resident_parent : E; }
+
 lbm_status run_resident(Engine* E, int64_t n_steps, int64_t mom_prev) {
-  StepBarrier* bar = static_cast<StepBarrier*>(E->bar.p);
-  CU(cudaMemsetAsync(&bar->error, 0, sizeof(int), E->stream));
+  Engine* H = halo_engine(E);
+  StepBarrier* bar = static_cast<StepBarrier*>(H->bar.p);
+  if (!H->bar_used) CU(cudaMemsetAsync(&bar->error, 0, sizeof(int), E->stream));
   const int* scratch = static_cast<const int*>(E->seg_scratch.p);
   while (n_steps > 0) {
     const bool last = n_steps <= 2 * kMaxResidentSteps;
     const int64_t n = last ? n_steps : kMaxResidentSteps;
-    if ((uint64_t)E->halo_epoch + (uint64_t)n + 2 >= (1ull << 32)) {  // tags would wrap: start afresh
-      CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));
-      E->halo_epoch = 1;
+    if ((uint64_t)H->halo_epoch + (uint64_t)n + 2 >= (1ull << 32)) {  // tags would wrap: start afresh
+      CU(cudaMemsetAsync(H->halo.p, 0, H->halo.cap, E->stream));
+      H->halo_epoch = 1;
     }
-    const unsigned epoch0 = E->halo_epoch;
-    E->halo_epoch += (unsigned)n + 1;
+    const unsigned epoch0 = H->halo_epoch;
+    H->halo_epoch += (unsigned)n + 1;
     CU(launch_stream_collide_resident(E->precision, E->features, static_cast<const LatticeView*>(E->L.views.p),
                                       static_cast<const SegRef*>(E->segs.p), static_cast<const int*>(E->n_segs.p),
                                       static_cast<const int*>(E->L.seg_word_off.p), scratch,
-                                      scratch + E->L.total_seg_words, E->rshape, E->halo.p, E->halo_cap, epoch0,
+                                      scratch + E->L.total_seg_words, E->rshape, H->halo.p, H->halo_cap, epoch0,
                                       (int)n, last ? (int)mom_prev : -1, &bar->error, E->stream));
     n_steps -= n;
     mom_prev = mom_prev < 0 ? -1 : mom_prev - n;
   }
-  E->bar_used = true;
+  H->bar_used = true;
   DEBUG_SYNC(E, "resident steps");
   return LBM_OK;
 }
 
 StepConfig resident_config(const Engine* E) {
   StepConfig c{};
-  c.warps_per_block = (E->rshape.own + 1) / 2;  // in the terms of the other shapes: two segments a warp
+  // in the terms of the other shapes: two segments a warp
+  c.warps_per_block = E->rshape.per_warp ? (E->rshape.own + 1) / 2 : E->rshape.warps;
   c.grid = E->rshape.grid;
   c.persistent = 2;
   c.cells_per_thread = 2;
@@ -1058,7 +1063,7 @@ lbm_status rebuild_worklist(Engine* E) {
                            static_cast<int*>(E->n_segs.p), E->stream));
   CU(launch_count_fluid(static_cast<const LatticeView*>(E->L.views.p), static_cast<const int*>(E->L.word_off.p),
                         E->n(), E->L.total_words, static_cast<unsigned long long*>(E->fluid_dev.p), E->stream));
-  if (!E->in_group) {
+  if (!E->in_group || E->resident_parent) {
     CU(cudaMemcpyAsync(E->h_nseg, E->n_segs.p, sizeof(int), cudaMemcpyDeviceToHost, E->stream));
     E->nseg_copied = true;
   }
@@ -1108,34 +1113,42 @@ lbm_status ensure_pairs(Engine* E) {
 }
 
 void take_seg_count(Engine* E) {
+  for (Engine* g : E->groups) take_seg_count(g);
   if (!E->nseg_copied) return;
   E->nseg_copied = false;
   E->seg_bound = *E->h_nseg;
 }
 
-lbm_status resident_prepare(Engine* E, bool* ok) {
+lbm_status resident_prepare(Engine* E, bool* ok, int max_own) {
   *ok = false;
   if (E->n() == 0 || debug_sync()) return LBM_OK;
-  if (E->nseg_copied && E->seg_bound > (long long)kResidentMaxOwn * E->sm_count) {  // the bound is too wide: count
+  const long long room = (long long)max_own * E->sm_count;
+  // the bound may be too wide for the faster kernel, or for either: count
+  if (E->nseg_copied && E->seg_bound > (long long)kResidentMaxOwn * E->sm_count) {
     CU(cudaStreamSynchronize(E->stream));
     take_seg_count(E);
   }
   const long long nseg = E->seg_bound;
-  if (nseg < 1 || nseg > (long long)kResidentMaxOwn * E->sm_count) return LBM_OK;
+  if (nseg < 1 || nseg > room) return LBM_OK;
   const int own = resident_own(nseg, E->sm_count);
   E->rshape.grid = (int)((nseg + own - 1) / own);
   const int most = (int)((nseg + E->rshape.grid - 1) / E->rshape.grid);  // segments of a block
-  E->rshape.per_warp = most <= kResidentMaxWarps ? 1 : 2;
-  E->rshape.warps = (most + E->rshape.per_warp - 1) / E->rshape.per_warp;
+  E->rshape.per_warp = most <= kResidentMaxWarps ? 1 : most <= kResidentMaxOwn ? 2 : 0;
+  if (E->rshape.per_warp) {
+    E->rshape.warps = (most + E->rshape.per_warp - 1) / E->rshape.per_warp;
+  } else {
+    E->rshape.warps = kResidentManyWarps;
+  }
   E->rshape.own = most;
-  if (E->halo_cap < nseg) {
+  Engine* H = halo_engine(E);
+  if (H->halo_cap < nseg) {
     // the whole word space if that is small: an exchange seldom makes the list outgrow it
-    const long long cap = std::min<long long>(E->L.total_seg_words, (long long)kResidentMaxOwn * E->sm_count);
+    const long long cap = std::min<long long>(E->L.total_seg_words, room);
     bool moved = false;
-    CU(E->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap)), &moved));
-    CU(cudaMemsetAsync(E->halo.p, 0, E->halo.cap, E->stream));  // no tag in it may match a future one
-    E->halo_epoch = 1;
-    E->halo_cap = (int)std::max(nseg, cap);
+    CU(H->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap)), &moved));
+    CU(cudaMemsetAsync(H->halo.p, 0, H->halo.cap, E->stream));  // no tag in it may match a future one
+    H->halo_epoch = 1;
+    H->halo_cap = (int)std::max(nseg, cap);
   }
   *ok = true;
   return LBM_OK;
@@ -1277,6 +1290,49 @@ void fill_result(Engine* E, int i, lbm_solve_result* out) {
 // 62.2 GLUPS; FP32 at 28 / 42 MB: 77.1 / 79.0).  32-48 candidates at a
 // time step 1.5x faster (FP32) than all 256, which stream from DRAM.
 // LBM_GROUPS=0 turns grouping off; LBM_GROUP_BYTES sets the budget (tests).
+//
+// Before that, groups that fit the chip: a batch of more segments than the
+// resident kernel holds is split into as few groups as hold them (first fit,
+// the largest members first), each stepped on the chip for the whole solve,
+// one after the other.  256 candidates, 17 groups of up to 17,632 segments,
+// time per step of all: FP32 61 us against 80 in L2-sized groups, BF16 65
+// against 95.  A batch with a member beyond the chip, or under an
+// LBM_GROUP_BYTES of its own, keeps to the L2-sized groups.
+// Solves of fewer than kGroupMinSteps steps step the batch as one set (loading
+// and storing a group costs about as much as ten of its steps).
+constexpr int kGroupMinSteps = 12;
+constexpr int kGroupOwn = kResidentManyOwn - 4;  // per SM; the rest is for what exchanges add
+
+bool group_bytes_set() { return std::getenv("LBM_GROUP_BYTES") != nullptr; }
+
+// The parts of such a split, or none.
+lbm_status resident_parts(Engine* E, std::vector<std::vector<Member*>>* parts) {
+  const int n = E->n(), total = E->L.total_seg_words;
+  std::vector<int> offs(total + 1);  // list index of every segment word
+  CU(cudaMemcpyAsync(offs.data(), static_cast<const int*>(E->seg_scratch.p) + total, sizeof(int) * (total + 1),
+                     cudaMemcpyDeviceToHost, E->stream));
+  CU(cudaStreamSynchronize(E->stream));
+  std::vector<int> count(n), order(n);
+  for (int i = 0; i < n; ++i) {
+    count[i] = offs[i + 1 < n ? E->L.h_swoff[i + 1] : total] - offs[E->L.h_swoff[i]];
+    order[i] = i;
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return count[a] > count[b]; });
+  const int room = kGroupOwn * E->sm_count;
+  if (count[order[0]] > room) return LBM_OK;
+  std::vector<int> filled, part_of(n);
+  for (int i : order) {
+    size_t k = 0;
+    while (k < filled.size() && filled[k] + count[i] > room) ++k;
+    if (k == filled.size()) filled.push_back(0);
+    filled[k] += count[i];
+    part_of[i] = (int)k;
+  }
+  parts->resize(filled.size());
+  for (int i = 0; i < n; ++i) (*parts)[part_of[i]].push_back(E->m[i]);
+  return LBM_OK;
+}
+
 bool groups_enabled() {
   static const bool on = [] {
     const char* e = std::getenv("LBM_GROUPS");
@@ -1285,17 +1341,13 @@ bool groups_enabled() {
   return on;
 }
 
-lbm_status ensure_groups(Engine* E) {
-  if (E->groups_decided) return LBM_OK;
-  E->groups_decided = true;
-  if (E->n() < 2 || E->fixed_grid || E->in_group || E->shape_fixed || !groups_enabled()) return LBM_OK;
+// The L2-sized parts; false: the batch steps as one set.
+bool l2_parts(Engine* E, std::vector<std::vector<Member*>>* out) {
+  std::vector<std::vector<Member*>>& parts = *out;
   double budget = 0.0;
   if (const char* e = std::getenv("LBM_GROUP_BYTES")) budget = std::atof(e);
   if (budget <= 0.0) {
-    int dev = 0, l2 = 0;
-    CU(cudaGetDevice(&dev));
-    CU(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
-    budget = l2 / 3.0 * (E->precision == LBM_F32 ? 1.0 : 2.0 / 3.0);
+    budget = E->l2_bytes / 3.0 * (E->precision == LBM_F32 ? 1.0 : 2.0 / 3.0);
   }
   const double sb = 9.0 * (double)storage_bytes(E->precision);
   double total = 0.0, largest = 0.0;
@@ -1303,8 +1355,7 @@ lbm_status ensure_groups(Engine* E) {
     total += sb * (double)m->fluid_cells;
     largest = std::max(largest, sb * (double)m->fluid_cells);
   }
-  if (total <= 1.5 * budget || largest > 0.25 * budget) return LBM_OK;
-  std::vector<std::vector<Member*>> parts(1);
+  if (total <= 1.5 * budget || largest > 0.25 * budget) return false;
   double acc = 0.0;
   for (Member* m : E->m) {
     const double b = sb * (double)m->fluid_cells;
@@ -1315,12 +1366,31 @@ lbm_status ensure_groups(Engine* E) {
     parts.back().push_back(m);
     acc += b;
   }
+  return true;
+}
+
+lbm_status ensure_groups(Engine* E) {
+  if (E->groups_decided) return LBM_OK;
+  E->groups_decided = true;
+  if (E->n() < 2 || E->fixed_grid || E->in_group || E->shape_fixed || !groups_enabled()) return LBM_OK;
+  std::vector<std::vector<Member*>> parts;
+  bool resident = false;
+  if (resident_enabled() && autotune_enabled() && !group_bytes_set() && !debug_sync()) {
+    lbm_status st = resident_parts(E, &parts);
+    if (st != LBM_OK) return st;
+    resident = parts.size() > 1;
+  }
+  if (!resident) {
+    parts.assign(1, {});
+    if (!l2_parts(E, &parts)) return LBM_OK;
+  }
   for (const auto& part : parts) {
     Engine* g = nullptr;
     lbm_status st = engine_new(E->precision, E->residual_every, E->stream, false, &g);
     if (st == LBM_OK) {
       g->own_members = false;
       g->in_group = true;
+      g->resident_parent = resident ? E : nullptr;
       E->groups.push_back(g);  // owned by E from here on
       st = engine_set_members(g, part);
     }
@@ -1342,7 +1412,7 @@ lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
   lbm_status st;
   bool resident = E->resident_now;
   if (E->step.persistent == 2 && !debug_sync()) {
-    if ((st = resident_prepare(E, &resident)) != LBM_OK) return st;
+    if ((st = resident_prepare(E, &resident, kResidentMaxOwn)) != LBM_OK) return st;
     if (!resident) E->step = shape(E, kStepWarps, kDefaultGridScale);  // the list outgrew the chip
   }
   if (resident && with_res && K > kMaxResidentSteps) {  // step T - K would not lie in the last launch
@@ -1372,11 +1442,12 @@ lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
 
 lbm_status enqueue_steps_and_reduce(Engine* E, int64_t n_steps, bool with_res) {
   lbm_status st;
-  E->bar_used = E->sweep_now;
+  E->bar_used = E->sweep_now;  // (its error word is cleared)
   {
     NvtxRange nvtx("lbm_time_steps");
     CU(cudaEventRecord(E->ev_begin, E->stream));
-    if (E->groups.empty()) {
+    const bool short_of_groups = !E->groups.empty() && E->groups[0]->resident_parent && n_steps < kGroupMinSteps;
+    if (E->groups.empty() || short_of_groups) {
       if ((st = enqueue_steps(E, n_steps, with_res)) != LBM_OK) return st;
     } else {
       for (Engine* g : E->groups)  // one group after the other: each stays in L2 for its steps
@@ -1409,15 +1480,26 @@ lbm_status enqueue_steps_and_reduce(Engine* E, int64_t n_steps, bool with_res) {
 // 2048 x 1024 tree 108 / 138).  It is the fastest shape everywhere it fits (us
 // per step, resident / best of the others): 128 x 64 T 0.93 / 1.29, 384 x 192
 // tree 1.18 / 1.43, half-domain collector 1.22 / 2.07, 1501 x 751 tree with
-// the Smagorinsky model 1.95 / 2.52, 2048 x 1024 tree 2.02 / 3.01.
+// the Smagorinsky model 1.95 / 2.52, 2048 x 1024 tree 2.02 / 3.01; with several
+// pairs of segments a warp, 1000 x 500 channels 3.1 / 3.5, 3000 x 1500 tree
+// 3.6 / 4.8, 995 x 561 obstacles with a zero-gradient outlet 4.1 / 7.5, the
+// narrowest margin 1400 x 700 in two channels 4.73 / 5.12, BF16 4.96 / 5.04.
 constexpr int64_t kResidentMinSteps = 8;
 
 lbm_status choose_resident(Engine* E, int64_t n_steps) {
   E->resident_now = false;
+  if (!E->groups.empty() && E->groups[0]->resident_parent) {
+    for (Engine* g : E->groups) {
+      lbm_status st = choose_resident(g, n_steps);
+      if (st != LBM_OK) return st;
+    }
+    return LBM_OK;
+  }
   if (E->shape_fixed || !E->groups.empty() || !resident_enabled() || !autotune_enabled() ||
       n_steps < kResidentMinSteps)
     return LBM_OK;
-  lbm_status st = resident_prepare(E, &E->resident_now);
+  lbm_status st =
+      resident_prepare(E, &E->resident_now, E->n() > 1 && group_bytes_set() ? kResidentMaxOwn : kResidentManyOwn);
   if (st == LBM_ERR_OOM) {  // no room for the halo words: the per-phase kernels need none
     cudaGetLastError();
     E->resident_now = false;
@@ -1504,12 +1586,14 @@ lbm_status enqueue_solve(Engine* E, int64_t n_steps) {
   if (cst == LBM_OK) cst = choose_sweep(E, n_steps);
   if (cst != LBM_OK) return cst;
   if (n_steps >= 256 && !E->resident_now && !E->sweep_now) {
+    const bool had = !E->groups.empty();
     lbm_status st = ensure_groups(E);
+    if (st == LBM_OK && !had && !E->groups.empty()) st = choose_resident(E, n_steps);
     if (st != LBM_OK) return st;
   }
   if (!E->groups.empty()) {
     for (Engine* g : E->groups)
-      if (!g->tuned && n_steps >= 256) {
+      if (!g->tuned && n_steps >= 256 && !g->resident_now) {
         lbm_status st = autotune(g);
         if (st != LBM_OK) return st;
       }
@@ -1552,6 +1636,11 @@ lbm_status enqueue_exchange(Engine* E, const std::vector<int>& which, const int3
   }
   for (int k = 0; k < nx_; ++k) E->seg_bound += n_swap[k];  // a new fluid cell opens at most one segment
   E->seg_bound = std::min<long long>(E->seg_bound, E->L.total_seg_words);
+  for (Engine* g : E->groups) {
+    for (int k = 0; k < nx_; ++k)
+      if (std::find(g->m.begin(), g->m.end(), E->m[which[k]]) != g->m.end()) g->seg_bound += n_swap[k];
+    g->seg_bound = std::min<long long>(g->seg_bound, g->L.total_seg_words);
+  }
   st = rebuild_worklist(E);
   if (st != LBM_OK) return st;
   CU(xfer(E->h_info, E->oc.info, sizeof(int) * 8 * nx_, cudaMemcpyDeviceToHost, E->stream));
@@ -1822,7 +1911,7 @@ lbm_status engine_set_step_config(Engine* E, int32_t warps_per_block, int32_t pe
   E->groups.clear();
   if (persistent == 2) {  // on-chip resident steps: the shape follows from the work-list
     bool ok = false;
-    lbm_status st = E->features ? LBM_OK : resident_prepare(E, &ok);
+    lbm_status st = E->features ? LBM_OK : resident_prepare(E, &ok, kResidentMaxOwn);
     if (st != LBM_OK) return st;
     if (!ok)
       return fail(LBM_ERR_ARG, "resident steps need plain BGK lattices whose segments fit in shared memory");

@@ -161,6 +161,7 @@ struct Engine {
   std::vector<Engine*> groups;
   bool groups_decided = false;
   bool in_group = false;  // this engine steps one group of another engine's members
+  Engine* resident_parent = nullptr;  // that engine, when the group was cut to fit the chip
   cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
   double step_ms = 0.0;
   int64_t step_launches = 0, fluid_updates = 0;
@@ -184,7 +185,7 @@ int engine_step_groups(const Engine* E);
 lbm_status rebuild_worklist(Engine* E);
 // Shape and halo buffer of a resident launch over the current work-list;
 // *ok: the set fits the chip.
-lbm_status resident_prepare(Engine* E, bool* ok);
+lbm_status resident_prepare(Engine* E, bool* ok, int max_own);
 // Whether the next n_steps of E step on the chip by rule (E->resident_now).
 lbm_status choose_resident(Engine* E, int64_t n_steps);
 // Take the work-list's length copied by the last rebuild (the stream has been

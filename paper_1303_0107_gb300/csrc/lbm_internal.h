@@ -199,10 +199,12 @@ int stream_collide_persistent_grid(int precision, int warps_per_block, int cells
 // ---- on-chip resident time steps (resident.cu) ------------------------------
 // A whole solve in one cooperative launch with the populations in shared
 // memory: block b of G owns segments [b n / G, (b+1) n / G) of the list
-// (at most kResidentMaxOwn), one or two per warp, and exchanges what its neighbours
-// need through a halo buffer of tagged words.
+// (at most kResidentMaxOwn with one or two per warp, at most kResidentManyOwn
+// with several pairs per warp), and exchanges what its neighbours need
+// through a halo buffer of tagged words.
 constexpr int kResidentMaxOwn = 48;
 constexpr int kResidentMaxWarps = 32;
+constexpr int kResidentManyOwn = 120, kResidentManyWarps = 20;
 // Segments per block of a resident launch over nseg: an equal share of every
 // SM, in whole groups of four, but not below 16 -- a step of a small list is
 // the chain from one block's published words to its neighbours' update, which
@@ -213,21 +215,21 @@ constexpr int kResidentMaxWarps = 32;
 // 2.02 / 1.98.
 __host__ __device__ inline int resident_own(long long nseg, int sm_count) {
   const long long share = ((nseg + sm_count - 1) / sm_count + 3) / 4 * 4;
-  return share < 16 ? 16 : share > kResidentMaxOwn ? kResidentMaxOwn : (int)share;
+  return share < 16 ? 16 : share > kResidentManyOwn ? kResidentManyOwn : (int)share;
 }
 struct ResidentShape {
   int grid;      // blocks
   int warps;     // warps per block
-  int per_warp;  // segments per warp, 1 or 2
+  int per_warp;  // segments per warp, 1 or 2; 0: pairs, several per warp
   int own;       // segments of the fullest block
 };
 // Bytes of a halo buffer for a list of that many segments.
 size_t resident_halo_bytes(int segments);
-// n_steps (even) time steps of a list of at most rs.per_warp rs.warps rs.grid segments;
+// n_steps (even) time steps of a list of at most rs.own rs.grid segments;
 // features: kernel build as in StepConfig; seg_flags / seg_offs: the
 // work-list build's per-word flags and their exclusive scan (the list index
 // of every segment word that holds fluid); halo: room for halo_cap segments,
-// tags epoch0 + 1 .. epoch0 + n_steps - 1 written by this launch (older tags
+// tags epoch0 .. epoch0 + n_steps - 1 written by this launch (older tags
 // must all be smaller); moments at the last step and at step mom_prev (-1:
 // none, else into the *_prev fields); *error is set when a wait gave up.
 cudaError_t launch_stream_collide_resident(int precision, int features, const LatticeView* views, const SegRef* segs,

@@ -198,16 +198,14 @@ struct alignas(16) PairInfo {  // of a warp's two slots
   int edge[16];   // lanes 0-5 (slot 0) and 8-13 (slot 1): (word << 2 | value) of W E NW NE SW SE; -1: none
 };
 
-// Fetch this warp's ghost words of step k into buffer `buf`; false: gave up.
+// Wait for the words that a warp's S slots read of other blocks at the step
+// tagged `want`: v[2 r] what the lane's upper neighbour of slot r sent down,
+// v[2 r + 1] what the lower one sent up, e the lane's edge word (words that
+// come from no other block are left unset); false: gave up.
 template <int S>
-__device__ __forceinline__ bool fetch_ghosts(float* buf, const PairInfo& pi, const HaloWord* halo, int parity,
-                                             unsigned want, int lane, int* error) {
-  const HaloWord* hb = halo + parity;
-  const int4 vt = *reinterpret_cast<const int4*>(pi.vert);
-  const int es = lane < 8 * S ? pi.edge[lane] : -1;
-  HaloWord v[2 * S], e;
+__device__ __forceinline__ bool poll_words(const HaloWord* hb, const int (&src)[4], int es, unsigned want, int lane,
+                                           int* error, HaloWord (&v)[2 * S], HaloWord& e) {
   const unsigned long long ready = (unsigned long long)want << 32;
-  const int src[4] = {vt.x, vt.y, vt.z, vt.w};
 #pragma unroll
   for (int u = 0; u < 2 * S; ++u) {
     v[u].hi = ready;
@@ -231,6 +229,18 @@ __device__ __forceinline__ bool fetch_ghosts(float* buf, const PairInfo& pi, con
       return false;
     }
   }
+  return true;
+}
+
+// Fetch this warp's ghost words of step k into buffer `buf`; false: gave up.
+template <int S>
+__device__ __forceinline__ bool fetch_ghosts(float* buf, const PairInfo& pi, const HaloWord* halo, int parity,
+                                             unsigned want, int lane, int* error) {
+  const int4 vt = *reinterpret_cast<const int4*>(pi.vert);
+  const int es = lane < 8 * S ? pi.edge[lane] : -1;
+  const int src[4] = {vt.x, vt.y, vt.z, vt.w};
+  HaloWord v[2 * S], e;
+  if (!poll_words<S>(halo + parity, src, es, want, lane, error, v, e)) return false;
   float* ga = buf + Layout<S>::kGhost0 + S * (threadIdx.x >> 5) * kGhostWords;
 #pragma unroll
   for (int u = 0; u < 2 * S; ++u)
@@ -589,20 +599,410 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
   }
 }
 
-template <class T, int S>
-void* resident_kernel(int features) {
-  switch (features) {
-    case 0: return (void*)k_stream_collide_resident<T, 0, S>;
-    case kFeatModels: return (void*)k_stream_collide_resident<T, kFeatModels, S>;
-    case kFeatMirror: return (void*)k_stream_collide_resident<T, kFeatMirror, S>;
-    case kFeatModels | kFeatMirror: return (void*)k_stream_collide_resident<T, kFeatModels | kFeatMirror, S>;
-    default: return nullptr;
+// ---- lists of more than kResidentMaxOwn segments per SM ----------------------
+//
+// One copy of the populations (AA pattern) and several pairs of segments per
+// warp.  Step k even reads every population where it lies after the last
+// collision -- slot i of the source cell, its own opposite slot beyond a wall
+// -- and writes the opposite population to the place just read; step k odd
+// finds what streamed to a cell in the cell's own slots (direction i in slot
+// opp(i)) and leaves its result there in place.  Every place is read and
+// written by one lane within a step, so one copy and the block's barrier
+// between steps do.  Source words come from a table in shared memory (two
+// slots' words to a register); odd steps need none.  What crosses to another
+// block is published and polled exactly as above, but goes from the polled
+// words to registers by shuffles; the lane's `remote` bits say where it
+// replaces the shared-memory value.  1.8 KB of shared memory per segment
+// against 4 KB, so up to kResidentManyOwn of them.
+//
+// Pairs that exchange come first in the slot order; half of the warps take
+// their pairs in reverse, so that words travel while other warps compute.
+//
+// What bounds it.  15 candidates (111 segments a block, three pairs a warp):
+// 3.45 us a step, per phase 5.6; without the exchange 3.3, without the
+// collisions as well 2.1 (the FMA pipe needs 1.2 for them).  Twenty warps of
+// 96 registers: 24 of 80 spill or, with one code for both kinds of step, run
+// 3.8; 16 of 128 take a fourth round, 4.3.  Always all twenty, though the last
+// round may be part empty: 52 segments a block 2.4 against 3.0 with thirteen
+// warps of two pairs.
+constexpr int kManyPairs = kResidentManyOwn / 2;
+struct ManyShared {
+  float rows[2 * kManyPairs][kSegWords];
+  float outside[32];                  // takes what leaves the block
+  uint4 src[kManyPairs][2][32];       // source words of directions 1-4 and 5-8: slot 2p low, 2p + 1 high half
+  SlotInfo slots[2 * kManyPairs];
+  PairInfo pairs[kManyPairs];
+  uint16_t remote[kManyPairs][32];    // directions that come from another block, slot 2p in the low byte
+};
+static_assert(sizeof(ManyShared) <= 227 * 1024, "shared memory of a block");
+static_assert((2 * kManyPairs * kSegWords + 32) <= 65536, "two slots' source words share a register");
+
+// What other blocks sent to slot r of the pair replaces what was read of it.
+__device__ __forceinline__ void take_words(float (&g)[9], const HaloWord& from_above, const HaloWord& from_below,
+                                           float edge, int r, unsigned remote, int lane) {
+  const int far = lane == 31 ? 1 : 0;
+  const float side = __shfl_sync(kFull, edge, 8 * r + far), above = __shfl_sync(kFull, edge, 8 * r + 2 + far),
+              below = __shfl_sync(kFull, edge, 8 * r + 4 + far);
+  const float a7 = __shfl_down_sync(kFull, halo_value(from_above, 1), 1);
+  const float a8 = __shfl_up_sync(kFull, halo_value(from_above, 2), 1);
+  const float b5 = __shfl_up_sync(kFull, halo_value(from_below, 1), 1);
+  const float b6 = __shfl_down_sync(kFull, halo_value(from_below, 2), 1);
+  if (remote & 1u) g[1] = side;
+  if (remote & 2u) g[2] = halo_value(from_below, 0);
+  if (remote & 4u) g[3] = side;
+  if (remote & 8u) g[4] = halo_value(from_above, 0);
+  if (remote & 16u) g[5] = lane == 0 ? below : b5;
+  if (remote & 32u) g[6] = lane == 31 ? below : b6;
+  if (remote & 64u) g[7] = lane == 31 ? above : a7;
+  if (remote & 128u) g[8] = lane == 0 ? above : a8;
+}
+
+__device__ __forceinline__ void source_words(const ManyShared& m, int p, int lane, unsigned (&src)[9]) {
+  asm volatile("" : "+r"(p));
+  const uint4 a = m.src[p][0][lane], b = m.src[p][1][lane];
+  src[1] = a.x, src[2] = a.y, src[3] = a.z, src[4] = a.w;
+  src[5] = b.x, src[6] = b.y, src[7] = b.z, src[8] = b.w;
+}
+
+// Step k of pair p, even or odd; false: a word did not come.
+template <class T, int FEAT, bool even>
+__device__ __forceinline__ bool many_step(ManyShared& m, int p, int k, int k_last, int mom_prev, unsigned epoch0,
+                                          unsigned tag_skew, HaloWord* halo, int parity, int lane, int* error) {
+  asm volatile("" : "+r"(lane));  // what follows from it is computed here, not kept over the loop: that spills
+  float* sm = m.rows[0];
+  const int own = 2 * p * kSegWords + lane;
+  const PairInfo& pi = m.pairs[p];
+  const SlotInfo* si = m.slots + 2 * p;
+  float g[2][9];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) g[r][0] = sm[own + r * kSegWords];
+  if (even) {
+    unsigned src[9];
+    source_words(m, p, lane, src);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      g[0][i] = sm[src[i] & 0xffffu];
+      g[1][i] = sm[src[i] >> 16];
+    }
+  } else {
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      g[0][i] = sm[own + opp_of(i) * 32];
+      g[1][i] = sm[own + kSegWords + opp_of(i) * 32];
+    }
+  }
+  const float4 par = *reinterpret_cast<const float4*>(pi.rho0);  // rho0 and omega of the slots
+  const int4 units = *reinterpret_cast<const int4*>(&pi.flags);
+  const unsigned flags = (unsigned)units.x;
+  if (flags & (kPublishes << 16 | kPublishes)) {  // warp-uniform
+    const int4 vt = *reinterpret_cast<const int4*>(pi.vert);
+    const int from[4] = {vt.x, vt.y, vt.z, vt.w};
+    const int es = lane < 16 ? pi.edge[lane] : -1;
+    const unsigned remote = m.remote[p][lane];
+    HaloWord v[4], e;
+    if (!poll_words<2>(halo + (even ? parity : 0), from, es, epoch0 + (unsigned)k + tag_skew, lane, error, v, e)) return false;
+    const float edge = halo_value(e, es & 3);
+    if (flags & kPublishes) take_words(g[0], v[0], v[1], edge, 0, remote, lane);
+    if (flags & kPublishes << 16) take_words(g[1], v[2], v[3], edge, 1, remote >> 8, lane);
+  }
+  if (flags & (kHasPort << 16 | kHasPort)) {
+    if (flags & kHasPort) ports_of(g[0], flags, si[0], par.x, lane);
+    if (flags & kHasPort << 16) ports_of(g[1], flags >> 16, si[1], par.y, lane);
+  }
+  float dr[2], ux[2], uy[2];
+  if ((FEAT & kFeatModels) && (flags & (kSlotModel << 16 | kSlotModel))) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const float rho0 = r ? par.y : par.x, omega = r ? par.w : par.z;
+      if (flags & kSlotModel << (16 * r))
+        collide_other(g[r], rho0, omega, si[r].L->collision, si[r].L->c_smag, dr[r], ux[r], uy[r]);
+      else
+        bgk(g[r], rho0, omega, dr[r], ux[r], uy[r]);
+    }
+  } else {
+    bgk2(g[0], g[1], f2(par.x, par.y), f2(par.z, par.w), dr[0], ux[0], uy[0], dr[1], ux[1], uy[1]);
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) round2<T>(g[0][i], g[1][i]);
+  if ((flags & (kPublishes << 16 | kPublishes)) && k != k_last) {
+    const unsigned tag = epoch0 + (unsigned)k + 1u;
+    HaloWord* out = halo + ((even ? 0 : parity) + lane);
+    if (flags & kPublishes) publish(out + units.y, flags, lane, g[0], tag);
+    if (flags & kPublishes << 16) publish(out + units.z, flags >> 16, lane, g[1], tag);
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) sm[own + r * kSegWords] = g[r][0];
+  if (even) {  // the place direction i came from takes the opposite one
+    unsigned src[9];
+    source_words(m, p, lane, src);  // read again: kept, they would spill
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      sm[src[i] & 0xffffu] = g[0][opp_of(i)];
+      sm[src[i] >> 16] = g[1][opp_of(i)];
+    }
+  } else {
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      sm[own + i * 32] = g[0][i];
+      sm[own + kSegWords + i * 32] = g[1][i];
+    }
+  }
+  if (k == k_last || k == mom_prev) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if ((si[r].fluid >> lane) & 1u) write_moments(si[r], lane, k == k_last, dr[r], ux[r], uy[r]);
+  }
+  return true;
+}
+
+// As k_stream_collide_resident.  Tags epoch0 .. epoch0 + n_steps - 1 are
+// published (the state before the first step goes the same way).
+template <class T, int FEAT>
+__global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
+    k_stream_collide_resident_many(const LatticeView* __restrict__ views, const SegRef* __restrict__ segs,
+                                   const int* __restrict__ n_segs, const int* __restrict__ seg_word_off,
+                                   const int* __restrict__ seg_flags, const int* __restrict__ seg_offs,
+                                   HaloWord* __restrict__ halo, int halo_cap, unsigned epoch0, int n_steps,
+                                   int mom_prev, int* __restrict__ error, unsigned tag_skew) {
+  extern __shared__ __align__(16) unsigned char many_smem[];
+  using P = Pop<T>;
+  ManyShared& m = *reinterpret_cast<ManyShared*>(many_smem);
+  const int nseg = n_segs[0];
+  int s0, s1;
+  block_range(nseg, gridDim.x, blockIdx.x, s0, s1);
+  const int n_own = s1 - s0;  // the host sizes the grid by a bound on nseg
+  if (n_own > 2 * kManyPairs) {
+    if (threadIdx.x == 0) atomicExch(error, 1);
+    return;
+  }
+  const int n_pairs = (n_own + 1) / 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+
+  // ---- once per launch: neighbours, slots, source words ----
+  // (scratch of this part lies where the rows go afterwards)
+  int(*s_nbq)[8] = reinterpret_cast<int(*)[8]>(m.rows);  // list index of each neighbouring segment, or -1
+  uint8_t* s_order = reinterpret_cast<uint8_t*>(s_nbq + 2 * kManyPairs);
+  uint8_t* s_slot = s_order + 2 * kManyPairs;
+  for (int i = threadIdx.x; i < 8 * n_own; i += blockDim.x) {
+    const SegRef sr = segs[s0 + (i >> 3)];
+    const int q = i & 7;
+    s_nbq[i >> 3][q] = list_index(views, seg_word_off, seg_flags, seg_offs, sr.lattice,
+                                  (sr.yw >> kSegWordBits) + pos_dy(q),
+                                  (sr.yw & ((1 << kSegWordBits) - 1)) + pos_dw(q));
+  }
+  __syncthreads();
+  auto is_remote = [&](int q) { return q >= 0 && (q < s0 || q >= s1); };
+  constexpr int kParts = (kResidentManyOwn + 31) / 32;
+  if (warp == 0) {  // slots: ports beside others, then those that exchange, then the rest (as above)
+    unsigned port[kParts], touch[kParts];
+#pragma unroll
+    for (int h = 0; h < kParts; ++h) {
+      const int t = lane + 32 * h;
+      bool remote = false, has_port = false;
+      if (t < n_own) {
+        for (int q = 0; q < 8; ++q) remote |= is_remote(s_nbq[t][q]);
+        const SegRef sr = segs[s0 + t];
+        const LatticeView& L = views[sr.lattice];
+        const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
+        const uint32_t fl = ~L.mask[(long long)y * mask_stride(L.wpr) + w];
+        has_port = (w == 0 && (fl & 1u)) || (w == (L.nx - 1) >> 5 && ((fl >> ((L.nx - 1) & 31)) & 1u));
+      }
+      port[h] = __ballot_sync(kFull, has_port);
+      touch[h] = __ballot_sync(kFull, remote && !has_port);
+    }
+    int n_port = 0, n_touch = 0;
+#pragma unroll
+    for (int h = 0; h < kParts; ++h) n_port += __popc(port[h]), n_touch += __popc(touch[h]);
+    const int mixed = min(n_port, n_own - n_port);  // pairs of a port and another segment
+    const unsigned below = (1u << lane) - 1u;
+    int ports = 0, touching = 0, plain = 0;  // of the parts before
+#pragma unroll
+    for (int h = 0; h < kParts; ++h) {
+      const int t = lane + 32 * h;
+      const unsigned own = t < n_own ? 1u << lane : 0u;
+      const unsigned all = n_own >= 32 * h + 32 ? kFull : n_own > 32 * h ? (1u << (n_own - 32 * h)) - 1u : 0u;
+      const unsigned rest = all & ~port[h] & ~touch[h];
+      const bool is_port = port[h] & own;
+      const int i = is_port ? ports + __popc(port[h] & below)
+                  : (touch[h] & own) ? touching + __popc(touch[h] & below) : n_touch + plain + __popc(rest & below);
+      if (own) {
+        const int j = i < mixed ? 2 * i + (is_port ? 0 : 1) : mixed + i;
+        s_order[j] = (uint8_t)t;
+        s_slot[t] = (uint8_t)j;
+      }
+      ports += __popc(port[h]);
+      touching += __popc(touch[h]);
+      plain += __popc(rest);
+    }
+  }
+  __syncthreads();
+  const uint16_t* __restrict__ nbs = segment_flags(segs, n_segs);
+  const int outside = 2 * kManyPairs * kSegWords + lane;  // takes what other blocks' cells get
+  for (int p = warp; p < n_pairs; p += n_warps) {
+    PairInfo& pi = m.pairs[p];
+    if (lane < 4) pi.vert[lane] = -1;
+    if (lane < 16) pi.edge[lane] = -1;
+    __syncwarp();
+    unsigned flags = 0, remote = 0;
+    unsigned off[8] = {};
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int j = 2 * p + r, base = j * kSegWords;
+      if (j >= n_own) {  // an empty slot relaxes a resting cell
+        if (lane == 0) {
+          pi.rho0[r] = 1.0f;
+          pi.omega[r] = 1.0f;
+          pi.unit0[r] = 0;
+          m.slots[j] = SlotInfo{-1, -1, 0.0f, 0, 0, views, 0u};
+        }
+#pragma unroll
+        for (int i = 1; i <= 8; ++i) off[i - 1] |= (unsigned)(base + i * 32 + lane) << (16 * r);
+        continue;
+      }
+      const int t = s_order[j], q = s0 + t;
+      const SegRef sr = segs[q];
+      const LatticeView& L = views[sr.lattice];
+      const int y = sr.yw >> kSegWordBits, w = sr.yw & ((1 << kSegWordBits) - 1);
+      const int x = (w << 5) + lane;
+      const uint32_t mc = L.mask[(long long)y * mask_stride(L.wpr) + w];
+      const bool fluid = !((mc >> lane) & 1u);
+      const bool inlet = x == 0, outlet = x == L.nx - 1;
+      const unsigned nb = nbs[(long long)q * 32 + lane];
+      const bool plane = (FEAT & kFeatMirror) && L.mirror && y == 0;  // the row next to the symmetry plane
+#pragma unroll
+      for (int i = 1; i <= 8; ++i) {
+        const int cx = cx_of(i);
+        int o = base + opp_of(i) * 32 + lane;  // bounce-back; nobody else's word beyond a port or in a solid cell
+        if (fluid && !(inlet && cx > 0) && !(outlet && cx < 0) && !((nb >> (opp_of(i) - 1)) & 1u)) {
+          const bool image = plane && (i == 5 || i == 6);  // see k_stream_collide_resident
+          const int si = image ? (i == 5 ? 8 : 7) : i;
+          const int sl = lane - cx, dy = image ? 0 : -cy_of(i);
+          const int dw = sl < 0 ? -1 : sl > 31 ? 1 : 0;
+          if (dy == 0 && dw == 0) {
+            o = base + si * 32 + sl;
+          } else {
+            const int nq = s_nbq[t][pos_of(dy, dw)];
+            if (is_remote(nq)) {
+              o = outside;
+              remote |= 1u << (i - 1 + 8 * r);
+            } else if (nq >= 0) {  // (a fluid source lies in a listed segment)
+              o = s_slot[nq - s0] * kSegWords + si * 32 + (sl & 31);
+            }
+          }
+        }
+        off[i - 1] |= (unsigned)o << (16 * r);
+      }
+      // what other blocks read of this segment, and what it reads of theirs
+      bool rem[8];
+#pragma unroll
+      for (int d = 0; d < 8; ++d) rem[d] = is_remote(s_nbq[t][d]);
+      const bool side = rem[0] || rem[2];
+      unsigned sf = 0;
+      if (rem[1] || rem[4] || rem[5]) sf |= kPubUp;
+      if (rem[3] || rem[6] || rem[7] || (plane && side)) sf |= kPubDown;
+      if (side) sf |= kPubSide;
+      auto word = [&](int d, int unit, int l, int value) {
+        return ((s_nbq[t][d] * 3 + unit) * kUnitWords + l) << 2 | value;
+      };
+      if (lane == 0) {
+        if (rem[1]) pi.vert[2 * r] = (s_nbq[t][1] * 3 + kUnitDown) * kUnitWords;
+        if (rem[3]) pi.vert[2 * r + 1] = (s_nbq[t][3] * 3 + kUnitUp) * kUnitWords;
+        if (rem[2]) pi.edge[8 * r + 0] = word(2, kUnitSide, 31, 0);
+        if (rem[0]) pi.edge[8 * r + 1] = word(0, kUnitSide, 0, 1);
+        if (rem[5]) pi.edge[8 * r + 2] = word(5, kUnitDown, 31, 2);
+        if (rem[4]) pi.edge[8 * r + 3] = word(4, kUnitDown, 0, 1);
+        if (rem[6]) pi.edge[8 * r + 4] = word(6, kUnitUp, 31, 1);
+        if (rem[7]) pi.edge[8 * r + 5] = word(7, kUnitUp, 0, 2);
+        if (plane && rem[2]) pi.edge[8 * r + 4] = word(2, kUnitDown, 31, 2);
+        if (plane && rem[0]) pi.edge[8 * r + 5] = word(0, kUnitDown, 0, 1);
+        pi.rho0[r] = L.rho0;
+        pi.omega[r] = L.omega;
+        pi.unit0[r] = q * 3 * kUnitWords;
+        const int ol = L.nx - 1 - (w << 5);
+        m.slots[j] = SlotInfo{w == 0 && !(mc & 1u) ? 0 : -1, ol < 32 && !((mc >> (ol & 31)) & 1u) ? ol : -1,
+                              w == 0 ? L.u_in[y] : 0.0f, L.port_scheme == LBM_PORTS_ZOU_HE,
+                              (long long)y * L.pitch + (w << 5), &L, ~mc};
+      }
+      if (__any_sync(kFull, fluid && (inlet || outlet))) sf |= kHasPort;
+      if (L.outlet_rule == LBM_OUT_NEUMANN) sf |= kNeumann;
+      if ((FEAT & kFeatModels) && L.collision != LBM_COLLIDE_BGK) sf |= kSlotModel;
+      flags |= sf << (16 * r);
+    }
+    m.src[p][0][lane] = make_uint4(off[0], off[1], off[2], off[3]);
+    m.src[p][1][lane] = make_uint4(off[4], off[5], off[6], off[7]);
+    m.remote[p][lane] = (uint16_t)remote;
+    if (lane == 0) pi.flags = flags;
+  }
+  __syncthreads();
+  // the canonical layout into the rows; what other blocks read of it goes out tagged epoch0
+  const int parity = halo_cap * 3 * kUnitWords;
+  for (int p = warp; p < n_pairs; p += n_warps) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const SlotInfo& si = m.slots[2 * p + r];
+      const unsigned sf = m.pairs[p].flags >> (16 * r);
+      const T* F = static_cast<const T*>(si.L->f) + si.row + lane;
+      const int pl = (int)si.L->plane;
+      float g[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        g[i] = (si.fluid >> lane) & 1u ? P::ld(F + (long long)i * pl) : 0.0f;
+        m.rows[2 * p + r][i * 32 + lane] = g[i];
+      }
+      if (sf & kPublishes) publish(halo + parity + m.pairs[p].unit0[r] + lane, sf, lane, g, epoch0);
+    }
+  }
+  // ---- the time steps ----
+  // this warp's pairs: n_mine of them (negative: a wait gave up) from `first` on, `stride` apart
+  int n_mine = n_pairs > warp ? (n_pairs - warp - 1) / n_warps + 1 : 0;
+  const bool reverse = (warp >> 2) & 1;
+  const int first = reverse ? warp + n_warps * (n_mine - 1) : warp, stride = reverse ? -n_warps : n_warps;
+  for (int k = 0; k < n_steps; k += 2) {
+    if ((k & 127) == 0) {
+      if (__syncthreads_or(n_mine < 0)) break;
+    } else {
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int j = 0, p = first; j < n_mine; ++j, p += stride)
+      if (!many_step<T, FEAT, true>(m, p, k, n_steps - 1, mom_prev, epoch0, tag_skew, halo, parity, lane, error))
+        n_mine = -1;
+    __syncthreads();
+#pragma unroll 1
+    for (int j = 0, p = first; j < n_mine; ++j, p += stride)
+      if (!many_step<T, FEAT, false>(m, p, k + 1, n_steps - 1, mom_prev, epoch0, tag_skew, halo, parity, lane, error))
+        n_mine = -1;
+  }
+  if (__syncthreads_or(n_mine < 0)) return;  // the global layout keeps the state from before the launch
+  // ---- the final state (an even number of steps) to the canonical layout ----
+  for (int j = warp; j < n_own; j += n_warps) {
+    const SlotInfo& si = m.slots[j];
+    if (!((si.fluid >> lane) & 1u)) continue;
+    T* F = static_cast<T*>(si.L->f) + si.row + lane;
+    const int pl = (int)si.L->plane;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) P::st(F + (long long)i * pl, m.rows[j][i * 32 + lane]);
+  }
+}
+
+template <class T, int FEAT>
+void* resident_kernel(int per_warp) {
+  switch (per_warp) {
+    case 1: return (void*)k_stream_collide_resident<T, FEAT, 1>;
+    case 2: return (void*)k_stream_collide_resident<T, FEAT, 2>;
+    default: return (void*)k_stream_collide_resident_many<T, FEAT>;
   }
 }
 
 template <class T>
 void* resident_kernel(int features, int per_warp) {
-  return per_warp == 1 ? resident_kernel<T, 1>(features) : resident_kernel<T, 2>(features);
+  switch (features) {
+    case 0: return resident_kernel<T, 0>(per_warp);
+    case kFeatModels: return resident_kernel<T, kFeatModels>(per_warp);
+    case kFeatMirror: return resident_kernel<T, kFeatMirror>(per_warp);
+    case kFeatModels | kFeatMirror: return resident_kernel<T, kFeatModels | kFeatMirror>(per_warp);
+    default: return nullptr;
+  }
 }
 
 void* resident_kernel_for(int precision, int features, int per_warp) {
@@ -627,10 +1027,15 @@ cudaError_t launch_stream_collide_resident(int precision, int features, const La
   // under the test hook every wait expects a tag that nobody writes
   unsigned tag_skew = barrier_timeout_test() ? 1u : 0u;
   if (!k || rs.grid < 1 || rs.warps < 1 ||
-      rs.warps > (rs.per_warp == 1 ? kResidentMaxWarps : kResidentMaxOwn / 2) || n_steps < 2 || (n_steps & 1) ||
+      rs.warps > (rs.per_warp == 1   ? kResidentMaxWarps
+                  : rs.per_warp == 2 ? kResidentMaxOwn / 2
+                                     : kResidentManyWarps) ||
+      rs.own > kResidentManyOwn || n_steps < 2 || (n_steps & 1) ||
       halo_cap < 1)
     return cudaErrorInvalidValue;
-  const int smem = 2 * (int)sizeof(float) * (rs.per_warp == 1 ? Layout<1>::kWords : Layout<2>::kWords);
+  const int smem = rs.per_warp == 1   ? 2 * (int)sizeof(float) * Layout<1>::kWords
+                   : rs.per_warp == 2 ? 2 * (int)sizeof(float) * Layout<2>::kWords
+                                      : (int)sizeof(ManyShared);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&views, (void*)&segs, (void*)&n_segs, (void*)&seg_word_off, (void*)&seg_flags,
