@@ -119,13 +119,11 @@ lbm_status lbm_load_state(lbm_handle h, const void* pops, size_t bytes, int src_
   (void)src_is_device;
   Engine* E = h->e;
   Member* m = E->m[0];
-  const size_t nx = m->nx, ny = m->ny, ncell = nx * ny;
+  const size_t nx = m->nx, ncell = nx * m->ny;
   const size_t sb = storage_bytes(E->precision);
   if (bytes < 9 * ncell * sb) return fail(LBM_ERR_ARG, "pops too small");
-  for (int i = 0; i < 9; ++i)
-    CU(xfer2d(static_cast<char*>(m->f) + i * m->plane * sb, (size_t)m->pitch * sb,
-                         static_cast<const char*>(pops) + i * ncell * sb, nx * sb, nx * sb, ny,
-                         cudaMemcpyDefault, E->stream));
+  CU(copy_planes({m->f, pops, m->plane * sb, (size_t)m->pitch * sb, ncell * sb, nx * sb, nx * sb, 9, m->ny},
+                 cudaMemcpyDefault, E->stream));
   CU(cudaStreamSynchronize(E->stream));
   return LBM_OK;
 }

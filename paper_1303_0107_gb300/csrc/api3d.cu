@@ -281,8 +281,11 @@ lbm_status select3(lbm3d_handle h, const float* drho, const float* ux, const flo
 
 lbm_status copy_field(lbm3d_handle h, const void* src, size_t src_pitch_bytes, size_t row_bytes, size_t rows,
                       void* dst, int dst_is_device) {
-  CU3(cudaMemcpy2DAsync(dst, row_bytes, src, src_pitch_bytes, row_bytes, rows,
-                        dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+  if (dst_is_device)
+    CU3(copy_planes({dst, src, 0, row_bytes, 0, src_pitch_bytes, row_bytes, 1, (int)rows}, cudaMemcpyDeviceToDevice,
+                    h->stream));
+  else
+    CU3(cudaMemcpy2DAsync(dst, row_bytes, src, src_pitch_bytes, row_bytes, rows, cudaMemcpyDeviceToHost, h->stream));
   CU3(cudaStreamSynchronize(h->stream));
   return LBM_OK;
 }
@@ -571,8 +574,11 @@ lbm_status lbm3d_load_state(lbm3d_handle h, const void* pops, size_t bytes, int 
   const View3& v = h->v;
   if (bytes != (size_t)kQ3 * h->ncells * h->elem) return fail(LBM_ERR_ARG, "pops has the wrong size");
   const size_t rows = (size_t)kQ3 * v.nz * v.ny;
-  CU3(cudaMemcpy2DAsync(v.f, (size_t)v.nxp * h->elem, pops, (size_t)v.nx * h->elem, (size_t)v.nx * h->elem, rows,
-                        src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
+  const size_t pitch = (size_t)v.nxp * h->elem, width = (size_t)v.nx * h->elem;
+  if (src_is_device)
+    CU3(copy_planes({v.f, pops, 0, pitch, 0, width, width, 1, (int)rows}, cudaMemcpyDeviceToDevice, h->stream));
+  else
+    CU3(cudaMemcpy2DAsync(v.f, pitch, pops, width, width, rows, cudaMemcpyHostToDevice, h->stream));
   CU3(cudaStreamSynchronize(h->stream));
   return LBM_OK;
 }

@@ -64,6 +64,31 @@ cudaError_t xfer2d(void* dst, size_t dpitch, const void* src, size_t spitch, siz
   return e;
 }
 
+namespace {
+bool on_this_device(const void* p) {
+  cudaPointerAttributes a{};
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+}  // namespace
+
+cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream) {
+  // (a launch takes fewer than 2^31 pieces of at least 128 bytes)
+  const bool fits = (c.width / 128 + 1) * (size_t)c.rows * (size_t)c.planes < (size_t)1 << 31;
+  if (fits && on_this_device(c.dst) && on_this_device(c.src)) return launch_copy_planes(c, stream);
+  for (int k = 0; k < c.planes; ++k) {
+    const cudaError_t e = xfer2d(static_cast<char*>(c.dst) + k * c.dst_plane, c.dst_pitch,
+                                 static_cast<const char*>(c.src) + k * c.src_plane, c.src_pitch, c.width,
+                                 (size_t)c.rows, kind, stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 void transfer_bytes(uint64_t* h2d, uint64_t* d2h) {
   if (h2d) *h2d = g_h2d.load();
   if (d2h) *d2h = g_d2h.load();
@@ -1000,7 +1025,7 @@ Engine::~Engine() {
   for (GrowBuf* b : {&L.views, &L.word_off, &L.seg_word_off, &XL.views, &XL.word_off, &XL.seg_word_off, &segs,
                      &n_segs, &seg_scratch, &partials, &result, &fluid_dev, &n_swap_dev, &dense_f, &oc_buf, &bar,
                      &best, &halo, &cell_list, &cell_scan, &pair_list, &pair_scan,
-                     &sweep_buf, &second})
+                     &sweep_buf, &second, &fill_list})
     b->release();
   if (h_bar_error) cudaFreeHost(h_bar_error);
   if (h_result) cudaFreeHost(h_result);
@@ -1142,8 +1167,8 @@ lbm_status resident_prepare(Engine* E, bool* ok, int max_own) {
   E->rshape.own = most;
   Engine* H = halo_engine(E);
   if (H->halo_cap < nseg) {
-    // the whole word space if that is small: an exchange seldom makes the list outgrow it
-    const long long cap = std::min<long long>(E->L.total_seg_words, room);
+    // some more than the list: an exchange seldom makes it outgrow that
+    const long long cap = std::min(std::min<long long>(E->L.total_seg_words, room), nseg + nseg / 4 + 1024);
     bool moved = false;
     CU(H->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap)), &moved));
     CU(cudaMemsetAsync(H->halo.p, 0, H->halo.cap, E->stream));  // no tag in it may match a future one
@@ -1206,12 +1231,28 @@ lbm_status engine_set_members(Engine* E, const std::vector<Member*>& members) {
   return LBM_OK;
 }
 
-lbm_status engine_reset(Engine* E) {
-  for (Member* mb : E->m) {
-    lbm_status st = member_reset(mb, E->stream);
-    if (st != LBM_OK) return st;
+// All members at once (256 candidates: three runtime calls each took 4.4 ms).
+lbm_status members_reset(Engine* E) {
+  std::vector<FillEntry> list;
+  for (Member* m : E->m) {
+    list.push_back({m->mask_base, m->mask0_base, m->mask_bytes});
+    list.push_back({m->f, nullptr, 9 * m->plane * storage_bytes(m->p.precision)});
+    list.push_back({m->drho, nullptr, 5 * align_up(m->plane * 4)});
+    m->steps_done = 0;
   }
-  lbm_status st = rebuild_worklist(E);
+  CU(E->fill_list.reserve(sizeof(FillEntry) * list.size()));
+  CU(cudaMemcpyAsync(E->fill_list.p, list.data(), sizeof(FillEntry) * list.size(), cudaMemcpyHostToDevice, E->stream));
+  constexpr int kMost = 65535;  // blocks in y
+  for (size_t i = 0; i < list.size(); i += kMost)
+    CU(launch_fill_list(static_cast<const FillEntry*>(E->fill_list.p) + i, (int)std::min<size_t>(kMost, list.size() - i),
+                        E->stream));
+  return LBM_OK;
+}
+
+lbm_status engine_reset(Engine* E) {
+  lbm_status st = E->n() == 1 ? member_reset(E->m[0], E->stream) : members_reset(E);
+  if (st != LBM_OK) return st;
+  st = rebuild_worklist(E);
   if (st != LBM_OK) return st;
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long) * E->n(), cudaMemcpyDeviceToHost,
                      E->stream));
@@ -1854,6 +1895,10 @@ lbm_status engine_read(Engine* E, int i, uint32_t which, void* dst, size_t dst_b
   switch (which) {
     case LBM_FIELD_MASK:
       if (dst_bytes < ncell) return fail(LBM_ERR_ARG, "dst too small");
+      if (on_this_device(dst)) {
+        CU(launch_unpack_mask(m->mask, m->nx, m->ny, m->wpr, static_cast<uint8_t*>(dst), E->stream));
+        break;
+      }
       CU(launch_unpack_mask(m->mask, m->nx, m->ny, m->wpr, m->cells, E->stream));
       CU(xfer(dst, m->cells, ncell, cudaMemcpyDefault, E->stream));
       break;
@@ -1861,22 +1906,21 @@ lbm_status engine_read(Engine* E, int i, uint32_t which, void* dst, size_t dst_b
       if (dst_bytes < ncell * 4) return fail(LBM_ERR_ARG, "dst too small");
       CU(launch_rho_from_drho(m->drho, (float)m->p.rho0, m->mask, m->nx, m->ny, m->pitch, m->wpr,
                               static_cast<float*>(E->dense_f.p), E->stream));
-      CU(xfer(dst, E->dense_f.p, ncell * 4, cudaMemcpyDefault, E->stream));
+      CU(copy_planes({dst, E->dense_f.p, 0, 0, 0, 0, ncell * 4, 1, 1}, cudaMemcpyDefault, E->stream));
       break;
     case LBM_FIELD_DRHO:
     case LBM_FIELD_UX:
     case LBM_FIELD_UY: {
       if (dst_bytes < ncell * 4) return fail(LBM_ERR_ARG, "dst too small");
       const float* src = which == LBM_FIELD_DRHO ? m->drho : which == LBM_FIELD_UX ? m->ux : m->uy;
-      CU(xfer2d(dst, nx * 4, src, (size_t)m->pitch * 4, nx * 4, ny, cudaMemcpyDefault, E->stream));
+      CU(copy_planes({dst, src, 0, nx * 4, 0, (size_t)m->pitch * 4, nx * 4, 1, m->ny}, cudaMemcpyDefault,
+                     E->stream));
       break;
     }
     case LBM_FIELD_POPS:
       if (dst_bytes < 9 * ncell * sb) return fail(LBM_ERR_ARG, "dst too small");
-      for (int k = 0; k < 9; ++k)
-        CU(xfer2d(static_cast<char*>(dst) + k * ncell * sb, nx * sb,
-                             static_cast<const char*>(m->f) + k * m->plane * sb, (size_t)m->pitch * sb, nx * sb,
-                             ny, cudaMemcpyDefault, E->stream));
+      CU(copy_planes({dst, m->f, ncell * sb, nx * sb, m->plane * sb, (size_t)m->pitch * sb, nx * sb, 9, m->ny},
+                     cudaMemcpyDefault, E->stream));
       break;
     default:
       return fail(LBM_ERR_ARG, "which must be exactly one LBM_FIELD_* value");

@@ -140,6 +140,8 @@ struct Engine {
   GrowBuf pair_list, pair_scan;
   bool pairs_valid = false;
 
+  GrowBuf fill_list;  // what a batch's reset clears and restores
+
   // sweeps (sweep.cu): the row list with its scan buffers, valid until the
   // work-list is rebuilt, and the second population buffer
   GrowBuf sweep_buf, second;

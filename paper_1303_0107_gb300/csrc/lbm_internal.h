@@ -262,6 +262,27 @@ cudaError_t launch_build_sweep(const LatticeView& L, const SweepList& s, cudaStr
 cudaError_t launch_sweep(const LatticeView& L, const void* F, void* G, const SweepList& s, int grid, int* error,
                          cudaStream_t stream);
 
+// ---- copies (copy.cu) --------------------------------------------------------
+// planes x rows rows of `width` bytes; strides in bytes.  Device memory of the
+// current device on both sides.
+struct PlaneCopy {
+  void* dst;
+  const void* src;
+  size_t dst_plane, dst_pitch, src_plane, src_pitch, width;
+  int planes, rows;
+};
+cudaError_t launch_copy_planes(const PlaneCopy& c, cudaStream_t stream);
+struct FillEntry {
+  void* dst;
+  const void* src;  // nullptr: zeros
+  size_t bytes;
+};
+// list: device
+cudaError_t launch_fill_list(const FillEntry* list, int n, cudaStream_t stream);
+// A PlaneCopy by the kernel where both sides are device memory of the current
+// device, else by the runtime as a copy of that kind.
+cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream);
+
 // ---- geometry / work-list (worklist.cu) ------------------------------------
 cudaError_t launch_pack_mask(const uint8_t* cells, int nx, int ny, int wpr, uint32_t* mask,
                              cudaStream_t stream);
