@@ -262,6 +262,29 @@ cudaError_t launch_build_sweep(const LatticeView& L, const SweepList& s, cudaStr
 cudaError_t launch_sweep(const LatticeView& L, const void* F, void* G, const SweepList& s, int grid, int* error,
                          cudaStream_t stream);
 
+// Inclusive prefix sum over a block of 1024 threads (all call; sums: shared, 32).
+#ifdef __CUDACC__
+__device__ __forceinline__ int block_inclusive_scan(int v, int* sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) sums[warp] = incl;
+  __syncthreads();
+  int before = sums[lane];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += u;
+  }
+  before = __shfl_sync(0xffffffffu, before, warp > 0 ? warp - 1 : 0);
+  return incl + (warp > 0 ? before : 0);
+}
+#endif
+
 // ---- copies (copy.cu) --------------------------------------------------------
 // planes x rows rows of `width` bytes; strides in bytes.  Device memory of the
 // current device on both sides.

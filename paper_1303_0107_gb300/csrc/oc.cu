@@ -116,21 +116,25 @@ __global__ void k_oc_emit(const LatticeView* __restrict__ views, const int* __re
                           unsigned long long* __restrict__ key_f, int* __restrict__ idx_f,
                           unsigned long long* __restrict__ key_s, int* __restrict__ idx_s,
                           int* __restrict__ info) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  // eight threads a word, four bits each: along a horizontal wall every cell of a
+  // word is a candidate, one thread's chain of loads for them all took longest
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = tid >> 3;
   if (i >= total) return;
+  const uint32_t mine = 0xfu << (4 * (tid & 7)), before = (1u << (4 * (tid & 7))) - 1u;
   int l, y, w;
   word_of(views, word_off, n, i, l, y, w);
   const LatticeView* L = views + l;
   const int nx = L->nx, pitch = L->pitch;
   const double rho0 = L->rho0d, mu = L->mu;
   const WordMasks m = word_masks(L->mask, nx, L->ny, L->wpr, y, w, L->guard);
-  int of = off_f[i], os = off_s[i];
+  int of = off_f[i] + __popc(m.fluid_cand & before), os = off_s[i] + __popc(m.solid_cand & before);
   bool bad = false;
   // a field value, its index checked in the bounds-checked build (0 when outside)
   const long long plane = L->plane;
   (void)plane;
   auto fld = [&](const float* a, long long c) { return LBM_OK_IDX(c, plane) ? (double)a[c] : 0.0; };
-  uint32_t fc = m.fluid_cand;
+  uint32_t fc = m.fluid_cand & mine;
   while (fc) {
     const int b = __ffs(fc) - 1;
     fc &= fc - 1;
@@ -145,7 +149,7 @@ __global__ void k_oc_emit(const LatticeView* __restrict__ views, const int* __re
     idx_f[of] = y * nx + x;
     ++of;
   }
-  uint32_t sc = m.solid_cand;
+  uint32_t sc = m.solid_cand & mine;
   while (sc) {
     const int b = __ffs(sc) - 1;
     sc &= sc - 1;
@@ -154,11 +158,11 @@ __global__ void k_oc_emit(const LatticeView* __restrict__ views, const int* __re
     // fluid 4-neighbours in the order E, N, W, S
     const bool fe = !((m.e >> b) & 1u), fn = !((m.n >> b) & 1u), fw = !((m.w >> b) & 1u),
                fs = !((m.s >> b) & 1u);
-    double sigma = 0.0;
-    if (fe) sigma = __dadd_rn(sigma, __ddiv_rn(__dmul_rn(mu, fabs(fld(L->uy, c + 1))), 0.5));
-    if (fn) sigma = __dadd_rn(sigma, __ddiv_rn(__dmul_rn(mu, fabs(fld(L->ux, c + pitch))), 0.5));
-    if (fw) sigma = __dadd_rn(sigma, __ddiv_rn(__dmul_rn(mu, fabs(fld(L->uy, c - 1))), 0.5));
-    if (fs) sigma = __dadd_rn(sigma, __ddiv_rn(__dmul_rn(mu, fabs(fld(L->ux, c - pitch))), 0.5));
+    double sigma = 0.0;  // (times 2 is what the division by 0.5 gives, exactly)
+    if (fe) sigma = __dadd_rn(sigma, __dmul_rn(__dmul_rn(mu, fabs(fld(L->uy, c + 1))), 2.0));
+    if (fn) sigma = __dadd_rn(sigma, __dmul_rn(__dmul_rn(mu, fabs(fld(L->ux, c + pitch))), 2.0));
+    if (fw) sigma = __dadd_rn(sigma, __dmul_rn(__dmul_rn(mu, fabs(fld(L->uy, c - 1))), 2.0));
+    if (fs) sigma = __dadd_rn(sigma, __dmul_rn(__dmul_rn(mu, fabs(fld(L->ux, c - pitch))), 2.0));
     bad |= isnan(sigma);
     key_s[os] = ~order_key(sigma);  // ascending key = descending sigma
     idx_s[os] = y * nx + x;
@@ -168,7 +172,13 @@ __global__ void k_oc_emit(const LatticeView* __restrict__ views, const int* __re
 }
 
 constexpr int kSelThreads = 1024;
+constexpr int kSelUnroll = 4;  // keys a thread has in flight
 
+// What bounds it: the chain of passes over the candidates and barriers.  An
+// exchange of 20 cells on 128 x 64, with its work-list: 54 us, 69 with all
+// twelve digits, a serial search of the 256 bins and one thread's run of
+// candidates in the compaction; 300 cells on the 2048 x 1024 tree 168 / 201;
+// 2000 cells on 4000 x 2000 channels 413 / 457.
 // Grid (2, lattices): block (0, l) selects among lattice l's fluid candidates,
 // block (1, l) among its solid candidates: the n smallest (key, idx) pairs,
 // written in candidate (= ascending idx) order to the lattice's pick range.
@@ -183,7 +193,8 @@ __global__ void __launch_bounds__(kSelThreads)
   __shared__ unsigned long long s_key;
   __shared__ unsigned int s_idx;
   __shared__ int s_rem;
-  __shared__ int scan[kSelThreads];
+  __shared__ int s_done;
+  __shared__ int s_scan[32];
   const int tid = threadIdx.x;
   const int l = blockIdx.y;
   const LatticeView* L = views + l;
@@ -211,66 +222,105 @@ __global__ void __launch_bounds__(kSelThreads)
     s_key = 0;
     s_idx = 0;
     s_rem = n;  // rank (1-based) of the threshold among matching candidates
+    s_done = 0;
   }
   __syncthreads();
-  // 12 digits of 8 bits: 8 of the score key, then 4 of the index
+  // 12 digits of 8 bits: 8 of the score key, then 4 of the index.  The search ends
+  // at the digit whose bin is taken whole (the bits below are then free): after
+  // three or four digits where the scores differ.
   for (int d = 0; d < 12; ++d) {
     for (int k = tid; k < 256; k += kSelThreads) hist[k] = 0;
     __syncthreads();
     const unsigned long long pk = s_key;
     const unsigned int pi = s_idx;
-    for (int k = tid; k < ncand; k += kSelThreads) {
-      const unsigned long long kk = key[k];
-      const unsigned int ii = (unsigned int)idx[k];
-      int digit;
-      bool match;
-      if (d < 8) {
-        match = d == 0 || (kk >> (64 - 8 * d)) == (pk >> (64 - 8 * d));
-        digit = (int)((kk >> (56 - 8 * d)) & 0xffu);
-      } else {
-        const int dd = d - 8;
-        match = kk == pk && (dd == 0 || (ii >> (32 - 8 * dd)) == (pi >> (32 - 8 * dd)));
-        digit = (int)((ii >> (24 - 8 * dd)) & 0xffu);
+    for (int k0 = tid; k0 < ncand; k0 += kSelUnroll * kSelThreads) {
+      unsigned long long kk[kSelUnroll];
+#pragma unroll
+      for (int u = 0; u < kSelUnroll; ++u)
+        if (k0 + u * kSelThreads < ncand) kk[u] = key[k0 + u * kSelThreads];
+#pragma unroll
+      for (int u = 0; u < kSelUnroll; ++u) {
+        const int k = k0 + u * kSelThreads;
+        if (k >= ncand) break;
+        int digit;
+        bool match;
+        if (d < 8) {
+          match = d == 0 || (kk[u] >> (64 - 8 * d)) == (pk >> (64 - 8 * d));
+          digit = (int)((kk[u] >> (56 - 8 * d)) & 0xffu);
+        } else {
+          const unsigned int ii = (unsigned int)idx[k];
+          const int dd = d - 8;
+          match = kk[u] == pk && (dd == 0 || (ii >> (32 - 8 * dd)) == (pi >> (32 - 8 * dd)));
+          digit = (int)((ii >> (24 - 8 * dd)) & 0xffu);
+        }
+        if (match) atomicAdd(&hist[digit], 1);
       }
-      if (match) atomicAdd(&hist[digit], 1);
     }
     __syncthreads();
-    if (tid == 0) {
-      int rem = s_rem, b = 0;
-      while (b < 255 && hist[b] < rem) {
-        rem -= hist[b];
-        ++b;
+    if (tid < 32) {  // the bin of rank s_rem: eight bins a lane
+      int c[8], sum = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sum += c[k] = hist[8 * tid + k];
+      int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (tid >= o) incl += u;
       }
-      s_rem = rem;
-      if (d < 8)
-        s_key = pk | ((unsigned long long)b << (56 - 8 * d));
-      else
-        s_idx = pi | ((unsigned int)b << (24 - 8 * (d - 8)));
+      const int rank = s_rem;
+      __syncwarp();
+      if (incl >= rank && incl - sum < rank) {  // one lane
+        int rem = rank - (incl - sum), b = 8 * tid, here = 0;
+        bool found = false;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (!found) {
+            if (c[k] < rem) {
+              rem -= c[k];
+              ++b;
+            } else {
+              here = c[k];
+              found = true;
+            }
+          }
+        const bool whole = here == rem;
+        s_rem = rem;
+        s_done = whole;
+        if (d < 8) {
+          const int sh = 56 - 8 * d;
+          s_key = pk | (unsigned long long)b << sh | (whole ? (1ull << sh) - 1ull : 0ull);
+          if (whole) s_idx = 0xffffffffu;
+        } else {
+          const int sh = 24 - 8 * (d - 8);
+          s_idx = pi | (unsigned int)b << sh | (whole ? (1u << sh) - 1u : 0u);
+        }
+      }
     }
     __syncthreads();
+    if (s_done) break;  // (written again only past two barriers)
   }
   const unsigned long long tk = s_key;
   const unsigned int ti = s_idx;
   // ordered compaction of all (key, idx) <= (tk, ti): exactly n of them
-  const int per = (ncand + kSelThreads - 1) / kSelThreads;
-  const int begin = min(ncand, tid * per), end = min(ncand, begin + per);
+  // (a warp takes a run of candidates, 32 at a time)
+  const int lane = tid & 31, warp = tid >> 5;
+  const int per = ((ncand + kSelThreads - 1) / kSelThreads) * 32;
+  const int begin = min(ncand, warp * per), end = min(ncand, begin + per);
+  auto taken = [&](int k) {
+    if (k >= end) return false;
+    const unsigned long long kk = key[k];
+    return kk < tk || (kk == tk && (unsigned int)idx[k] <= ti);
+  };
   int cnt = 0;
-  for (int k = begin; k < end; ++k) {
-    const unsigned long long kk = key[k];
-    cnt += (kk < tk || (kk == tk && (unsigned int)idx[k] <= ti)) ? 1 : 0;
-  }
-  scan[tid] = cnt;
-  __syncthreads();
-  for (int off = 1; off < kSelThreads; off <<= 1) {
-    const int v = tid >= off ? scan[tid - off] : 0;
-    __syncthreads();
-    scan[tid] += v;
-    __syncthreads();
-  }
-  int pos = scan[tid] - cnt;
-  for (int k = begin; k < end; ++k) {
-    const unsigned long long kk = key[k];
-    if (kk < tk || (kk == tk && (unsigned int)idx[k] <= ti)) sel[pos++] = idx[k];
+  for (int k = begin + lane; k - lane < end; k += 32) cnt += taken(k) ? 1 : 0;
+  // the prefix sum of the warp's last lane, less what the warp holds, is where its picks start
+  const int incl = block_inclusive_scan(cnt, s_scan);
+  int pos = __shfl_sync(0xffffffffu, incl - cnt, 0);
+  for (int k = begin + lane; k - lane < end; k += 32) {
+    const bool take = taken(k);
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (take) sel[pos + __popc(m & ((1u << lane) - 1u))] = idx[k];
+    pos += __popc(m);
   }
 }
 
@@ -332,7 +382,7 @@ cudaError_t launch_oc_select(const LatticeView* views, const int* word_off, int 
   count_launches(1);
   if ((e = launch_scan(s.cnt_f, s.off_f, total, s.scan_tmp, stream)) != cudaSuccess) return e;
   if ((e = launch_scan(s.cnt_s, s.off_s, total, s.scan_tmp, stream)) != cudaSuccess) return e;
-  k_oc_emit<<<blocks_for(total, 256), 256, 0, stream>>>(views, word_off, n_lattices, total, s.off_f,
+  k_oc_emit<<<blocks_for(8ll * total, 256), 256, 0, stream>>>(views, word_off, n_lattices, total, s.off_f,
                                                         s.off_s, s.key_f, s.idx_f, s.key_s, s.idx_s,
                                                         s.info);
   k_oc_select<<<dim3(2, n_lattices), kSelThreads, 0, stream>>>(views, word_off, s.key_f, s.idx_f, s.key_s,

@@ -77,6 +77,9 @@ __global__ void __launch_bounds__(kRedThreads)
   const int n_outlets = L->n_outlets;
   const double rho0 = L->rho0d;
   const int wl = (nx - 1) >> 5, bl = (nx - 1) & 31;
+  __shared__ double s_partials[2 * kResidualBlocks];  // one thread adds them up below, in order
+  if (with_residual)
+    for (int k = threadIdx.x; k < 2 * kResidualBlocks; k += kRedThreads) s_partials[k] = partials[k];
   double s_in = 0.0, s_out = 0.0, m_in = 0.0, n_in = 0.0, n_out = 0.0;
   for (int y = threadIdx.x; y < ny; y += kRedThreads) {
     const uint32_t* mr = L->mask + (long long)y * mask_stride(wpr);
@@ -137,8 +140,8 @@ __global__ void __launch_bounds__(kRedThreads)
     double res = -1.0, sdu = 0.0, su = 0.0;
     if (with_residual) {
       for (int b = 0; b < kResidualBlocks; ++b) {
-        sdu += partials[2 * b];
-        su += partials[2 * b + 1];
+        sdu += s_partials[2 * b];
+        su += s_partials[2 * b + 1];
       }
       res = sdu / su;
     }

@@ -126,27 +126,20 @@ __global__ void k_count_fluid(const LatticeView* __restrict__ views, const int* 
 // Used for small inputs and for the top level of the multi-block scan.
 __global__ void __launch_bounds__(1024) k_scan_chunked(const int* __restrict__ in, int* __restrict__ out,
                                                        int n) {
-  __shared__ int sums[1024];
+  __shared__ int sums[32];
   const int tid = threadIdx.x;
   const int per = (n + 1023) / 1024;
   const int begin = min(n, tid * per), end = min(n, begin + per);
   int s = 0;
   for (int i = begin; i < end; ++i) s += in[i];
-  sums[tid] = s;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    const int v = tid >= off ? sums[tid - off] : 0;
-    __syncthreads();
-    sums[tid] += v;
-    __syncthreads();
-  }
-  int run = sums[tid] - s;  // exclusive prefix of this chunk
+  const int incl = block_inclusive_scan(s, sums);
+  int run = incl - s;  // exclusive prefix of this chunk
   for (int i = begin; i < end; ++i) {
     const int v = in[i];
     out[i] = run;
     run += v;
   }
-  if (tid == 1023) out[n] = sums[1023];
+  if (tid == 1023) out[n] = incl;
 }
 
 constexpr int kScanThreads = 256;
