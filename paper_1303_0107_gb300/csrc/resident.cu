@@ -10,7 +10,8 @@
 // SMs (the 2048 x 1024 distributor: 6976 segments, 5.75 MB of FP32
 // populations, against 152 x 227 KB) is split into contiguous ranges of its
 // segment list, one range per block (at most kResidentMaxOwn segments, one
-// block per SM, all blocks resident: a cooperative launch).  A block keeps
+// block per SM, all blocks resident: a cooperative launch; longer lists, up to
+// kResidentManyOwn a block, in a kernel of their own below).  A block keeps
 // its segments' nine population rows as FP32 in two step buffers in shared
 // memory (read one, write the other, a plain pull scheme; 16-bit storage
 // rounds every value to its type before it is stored, so the values are
