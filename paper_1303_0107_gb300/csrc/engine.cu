@@ -1169,8 +1169,8 @@ lbm_status resident_prepare(Engine* E, bool* ok, int max_own) {
   if (H->halo_cap < nseg) {
     // some more than the list: an exchange seldom makes it outgrow that
     const long long cap = std::min(std::min<long long>(E->L.total_seg_words, room), nseg + nseg / 4 + 1024);
-    bool moved = false;
-    CU(H->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap)), &moved));
+    H->halo_cap = 0;  // a growth that fails has freed the buffer
+    CU(H->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap))));
     CU(cudaMemsetAsync(H->halo.p, 0, H->halo.cap, E->stream));  // no tag in it may match a future one
     H->halo_epoch = 1;
     H->halo_cap = (int)std::max(nseg, cap);
@@ -1534,6 +1534,8 @@ lbm_status choose_resident(Engine* E, int64_t n_steps) {
       lbm_status st = choose_resident(g, n_steps);
       if (st != LBM_OK) return st;
     }
+    // a later group's growth that failed took the buffer of the earlier ones with it
+    for (Engine* g : E->groups) g->resident_now &= g->seg_bound <= E->halo_cap;
     return LBM_OK;
   }
   if (E->shape_fixed || !E->groups.empty() || !resident_enabled() || !autotune_enabled() ||

@@ -1032,7 +1032,7 @@ cudaError_t launch_stream_collide_resident(int precision, int features, const La
                   : rs.per_warp == 2 ? kResidentMaxOwn / 2
                                      : kResidentManyWarps) ||
       rs.own > kResidentManyOwn || n_steps < 2 || (n_steps & 1) ||
-      halo_cap < 1)
+      !halo || halo_cap < 1)
     return cudaErrorInvalidValue;
   const int smem = rs.per_warp == 1   ? 2 * (int)sizeof(float) * Layout<1>::kWords
                    : rs.per_warp == 2 ? 2 * (int)sizeof(float) * Layout<2>::kWords
