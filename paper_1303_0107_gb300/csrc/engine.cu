@@ -1234,18 +1234,20 @@ lbm_status engine_set_members(Engine* E, const std::vector<Member*>& members) {
 // All members at once (256 candidates: three runtime calls each took 4.4 ms).
 lbm_status members_reset(Engine* E) {
   std::vector<FillEntry> list;
+  size_t largest = 0;
   for (Member* m : E->m) {
     list.push_back({m->mask_base, m->mask0_base, m->mask_bytes});
     list.push_back({m->f, nullptr, 9 * m->plane * storage_bytes(m->p.precision)});
     list.push_back({m->drho, nullptr, 5 * align_up(m->plane * 4)});
-    m->steps_done = 0;
+    largest = std::max(largest, list[list.size() - 2].bytes);
   }
   CU(E->fill_list.reserve(sizeof(FillEntry) * list.size()));
   CU(cudaMemcpyAsync(E->fill_list.p, list.data(), sizeof(FillEntry) * list.size(), cudaMemcpyHostToDevice, E->stream));
   constexpr int kMost = 65535;  // blocks in y
   for (size_t i = 0; i < list.size(); i += kMost)
     CU(launch_fill_list(static_cast<const FillEntry*>(E->fill_list.p) + i, (int)std::min<size_t>(kMost, list.size() - i),
-                        E->stream));
+                        largest, E->sm_count, E->stream));
+  for (Member* m : E->m) m->steps_done = 0;
   return LBM_OK;
 }
 

@@ -300,8 +300,8 @@ struct FillEntry {
   const void* src;  // nullptr: zeros
   size_t bytes;
 };
-// list: device
-cudaError_t launch_fill_list(const FillEntry* list, int n, cudaStream_t stream);
+// list: device; largest: bytes of its largest entry
+cudaError_t launch_fill_list(const FillEntry* list, int n, size_t largest, int sm_count, cudaStream_t stream);
 // A PlaneCopy by the kernel where both sides are device memory of the current
 // device, else by the runtime as a copy of that kind.
 cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream);
