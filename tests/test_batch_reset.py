@@ -37,3 +37,14 @@ def test_large_members_reset_at_the_rate_of_their_handles():
     together = _fastest(two.reset)
     two.close()
     assert together < 1.4 * 2 * alone, (together, alone)
+
+
+def test_reset_succeeds_without_memory_for_its_list():
+    members = [dict(cells=I.channel(64 + 8 * i, 14), tau=0.8, u_max=0.02) for i in range(3)]
+    b = L.Batch(members, residual_every=0)
+    first = [r["dp"] for r in b.solve(40)]
+    L.lib.debug_fail_alloc(0)  # the next device allocation fails
+    b.reset()
+    L.lib.debug_fail_alloc(-1)
+    assert [r["dp"] for r in b.solve(40)] == first
+    b.close()
