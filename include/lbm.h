@@ -53,7 +53,8 @@ typedef enum {
   LBM_ERR_OOM = 3,       /* device or pinned host allocation failed */
   LBM_ERR_CUDA = 4,      /* a CUDA call failed; the handle must be destroyed */
   LBM_ERR_DIVERGED = 5,  /* a reduction or a score is not finite */
-  LBM_ERR_TIMEOUT = 6,   /* a bounded device-side wait gave up */
+  LBM_ERR_TIMEOUT = 6,   /* a bounded device-side wait gave up; after a solve: the state is void until
+                            lbm_reset or lbm_load_state, the handle stays usable */
   LBM_ERR_BUSY = 7,      /* resource temporarily unavailable (admission refused) */
   LBM_ERR_CANCELLED = 8  /* a served request withdrawn with lbm_server_cancel */
 } lbm_status;
@@ -293,7 +294,8 @@ void lbm_debug_fail_alloc(int64_t after);
  * called again with 0): the persistent step kernel's grid barriers then wait
  * for one arrival more than the grid makes, and the resident kernel's halo
  * polls for a step tag that nobody writes, so every wait gives up after its
- * poll limit (2^22 loads, a few seconds), the launch ends early and the
+ * poll limit (2^22 loads, a few seconds), and the sweeps take a copy that has
+ * arrived as one that has not; the launch ends early and the
  * solve returns LBM_ERR_TIMEOUT; the handle stays usable (lbm_reset or
  * lbm_load_state restores a state).  No device fault is involved.         */
 void lbm_debug_barrier_timeout(int32_t on);

@@ -269,11 +269,12 @@ __device__ __forceinline__ void run_step(const LatticeView& L, const Run& r, con
 // One sweep: kSteps time steps of the lattice L (its populations read through
 // the map `from`, the result written to G).  list: the rows of all tiles
 // holding fluid, n_rows their number, cost: see share_begin, states: of every
-// row of every tile.
+// row of every tile.  give_up: a block's wait for its input row of that number
+// or a later one counts as run out (the test hook; else larger than any).
 __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
     k_sweep(const __grid_constant__ LatticeView L, const __grid_constant__ CUtensorMap from, float* __restrict__ G,
             const int* __restrict__ list, const int* __restrict__ cost, const int* __restrict__ n_rows,
-            const RowState* __restrict__ states, int* __restrict__ error) {
+            const RowState* __restrict__ states, int* __restrict__ error, unsigned give_up) {
   extern __shared__ __align__(128) unsigned char sweep_smem[];
   __shared__ __align__(8) unsigned long long s_full[kRing0];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -305,9 +306,13 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
     int failed = 0;
     if (level > kSteps) {  // the warp that issues the copies and waits for them
       int copied = r_lo, arrived = r_lo;  // next input rows to copy and to wait for
+      auto wait_row = [&](int y) {
+        const unsigned i = seq + (unsigned)(y - r_lo);
+        return bar_wait(shared_addr(&s_full[i % kRing0]), (i / kRing0) & 1u) && i < give_up;
+      };
       for (int k = r.k_lo - 1; k <= r.k_hi; ++k) {
         // row i takes the place of row i - 8, last read in turn i - 7
-        for (; copied <= min(k + kRing0 - 2, r_hi); ++copied) {
+        for (; !failed && copied <= min(k + kRing0 - 2, r_hi); ++copied) {
           const unsigned slot = (seq + (unsigned)(copied - r_lo)) % kRing0;
           const unsigned bar = shared_addr(&s_full[slot]);
           if (lane == 0) {
@@ -316,12 +321,11 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
           }
         }
         // what the next turn reads has arrived before this one ends
-        for (; arrived <= min(k + 2, r_hi); ++arrived) {
-          const unsigned i = seq + (unsigned)(arrived - r_lo);
-          if (!failed && !bar_wait(shared_addr(&s_full[i % kRing0]), (i / kRing0) & 1u)) failed = 1;
-        }
+        for (; !failed && arrived <= min(k + 2, r_hi); ++arrived) failed = !wait_row(arrived);
         __syncthreads();
       }
+      if (failed)  // no copy is issued after the one that failed; those in flight land (or give up) before the block leaves
+        for (int y = arrived - 1; y < copied; ++y) (void)wait_row(y);
     } else {
       r.lag = 2 * (level - 1);
       r.lo = max(1, y_lo - (kSteps - level));
@@ -339,10 +343,8 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
         run_step<false, true>(L, r, in, nullptr, G, xs + col, col, window, lane, rho0, omega);
     }
     seq += (unsigned)(r_hi - r_lo + 1);
-    if (__syncthreads_or(failed)) {  // a copy never arrived: its place is never read again, the sweep is void
+    if (__syncthreads_or(failed)) {  // the sweep is void
       if (threadIdx.x == 0) atomicExch(error, 1);
-      if (threadIdx.x == kWarps * 32)  // wait (bounded) for what may still be in flight, then leave
-        for (int s = 0; s < kRing0; ++s) (void)bar_wait(shared_addr(&s_full[s]), 0u);
       return;
     }
   }
@@ -465,8 +467,9 @@ cudaError_t launch_sweep(const LatticeView& L, const void* F, void* G, const Swe
   CUtensorMap from;
   if (!population_map(&from, L, F)) return cudaErrorInvalidValue;
   float* g = static_cast<float*>(G);
+  unsigned give_up = barrier_timeout_test() ? kRing0 : 0xffffffffu;  // (the first row of a barrier's second phase)
   void* args[] = {(void*)&L, (void*)&from, (void*)&g, (void*)&sl.list, (void*)&sl.cost,
-                  (void*)&sl.n_rows, (void*)&sl.states, (void*)&error};
+                  (void*)&sl.n_rows, (void*)&sl.states, (void*)&error, (void*)&give_up};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
