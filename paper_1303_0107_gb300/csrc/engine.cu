@@ -420,7 +420,7 @@ lbm_status run_persistent(Engine* E, int64_t pairs) {
     CU(launch_stream_collide_persistent(E->precision, static_cast<const LatticeView*>(E->L.views.p),
                                         static_cast<const SegRef*>(E->segs.p),
                                         static_cast<const int*>(E->n_segs.p), (int)k, E->step,
-                                        static_cast<StepBarrier*>(E->bar.p), E->stream));
+                                        static_cast<StepBarrier*>(E->bar.p), !E->bar_used, E->stream));
     E->bar_used = true;
     pairs -= k;
   }
@@ -632,6 +632,7 @@ std::vector<long long> tune_key(const Engine* E) {
 lbm_status autotune(Engine* E) {
   NvtxRange nvtx("lbm_autotune");
   E->tuned = true;
+  E->bar_used = false;
   E->step = shape(E, kStepWarps, kDefaultGridScale);
   if (!autotune_enabled() || debug_sync()) return LBM_OK;
   const std::vector<long long> key = tune_key(E);

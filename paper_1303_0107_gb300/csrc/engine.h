@@ -114,7 +114,7 @@ struct Engine {
   unsigned long long* h_count = nullptr;  // pinned [n]
   int* h_nswap = nullptr;                 // pinned [n]
   int* h_bar_error = nullptr;             // pinned: grid-barrier error flag of the last solve
-  bool bar_used = false;                  // the last enqueued solve ran the persistent kernel
+  bool bar_used = false;                  // the error word was cleared for the solve being enqueued, which may set it
 
   // on-chip resident steps (step.persistent == 2): a host-side bound on the
   // segments of the current work-list (exact when the list was last counted,

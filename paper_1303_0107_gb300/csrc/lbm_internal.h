@@ -172,9 +172,9 @@ int stream_collide_pairs_blocks_per_sm(int precision, int phase, int moments, in
 struct StepBarrier {
   unsigned count;  // arrivals since the launch began
   unsigned gen;    // unused
-  int error;       // set when a wait gave up (the launch then stops early)
   int extra;       // arrivals awaited beyond the grid: 0, or 1 under the test hook
                    // (lbm_debug_barrier_timeout) so that every wait runs out
+  int error;       // set when a wait gave up (the launch then stops early)
 };
 // lbm_debug_barrier_timeout: the next persistent launches wait for an arrival
 // that never comes (the bounded-wait failure path, tested without a fault)
@@ -189,11 +189,12 @@ int stream_collide_blocks_per_sm(int precision, int phase, int moments, int warp
 // launch with a grid barrier between phases; sc.grid must not exceed
 // stream_collide_persistent_grid (every block resident at once), and
 // 2 * n_pairs * sc.grid must stay below 2^32.  The
-// barrier is reset on the stream first; a barrier wait that gives up sets
+// barrier is reset on the stream first, its error word only where `fresh` (the
+// first launch of a solve that may set it); a barrier wait that gives up sets
 // bar->error and ends the launch early.
 cudaError_t launch_stream_collide_persistent(int precision, const LatticeView* views, const SegRef* segs,
                                              const int* n_segs, int n_pairs, StepConfig sc, StepBarrier* bar,
-                                             cudaStream_t stream);
+                                             bool fresh, cudaStream_t stream);
 int stream_collide_persistent_grid(int precision, int warps_per_block, int cells_per_thread);
 
 // ---- on-chip resident time steps (resident.cu) ------------------------------

@@ -1304,14 +1304,13 @@ int stream_collide_persistent_grid(int precision, int warps_per_block, int cells
 
 cudaError_t launch_stream_collide_persistent(int precision, const LatticeView* views, const SegRef* segs,
                                              const int* n_segs, int n_pairs, StepConfig sc, StepBarrier* bar,
-                                             cudaStream_t stream) {
+                                             bool fresh, cudaStream_t stream) {
   void* k = persistent_kernel_for(precision, sc.cells_per_thread);
   if (!k || !shape_ok(sc) || sc.features || n_pairs < 1 ||
       sc.grid > stream_collide_persistent_grid(precision, sc.warps_per_block, sc.cells_per_thread) ||
       2ull * (unsigned long long)n_pairs * (unsigned long long)sc.grid >= (1ull << 32))
     return cudaErrorInvalidValue;
-  // a fresh barrier: count 0, no error
-  cudaError_t e = cudaMemsetAsync(bar, 0, sizeof(StepBarrier), stream);
+  cudaError_t e = cudaMemsetAsync(bar, 0, fresh ? sizeof(StepBarrier) : offsetof(StepBarrier, error), stream);
   if (e != cudaSuccess) return e;
   if (barrier_timeout_test() &&
       (e = cudaMemsetAsync(reinterpret_cast<char*>(bar) + offsetof(StepBarrier, extra), 1, 1, stream)) != cudaSuccess)
