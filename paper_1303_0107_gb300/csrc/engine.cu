@@ -1145,6 +1145,13 @@ void take_seg_count(Engine* E) {
   E->seg_bound = *E->h_nseg;
 }
 
+void set_halo_room(Engine* E, size_t bytes) {
+  E->halo_room = bytes;
+  if (E->halo.cap <= bytes) return;
+  E->halo.release();
+  E->halo_cap = 0;
+}
+
 lbm_status resident_prepare(Engine* E, bool* ok, int max_own) {
   *ok = false;
   if (E->n() == 0 || debug_sync()) return LBM_OK;
@@ -1169,12 +1176,15 @@ lbm_status resident_prepare(Engine* E, bool* ok, int max_own) {
   Engine* H = halo_engine(E);
   if (H->halo_cap < nseg) {
     // some more than the list: an exchange seldom makes it outgrow that
-    const long long cap = std::min(std::min<long long>(E->L.total_seg_words, room), nseg + nseg / 4 + 1024);
+    long long cap = std::max(nseg, std::min(std::min<long long>(E->L.total_seg_words, room), nseg + nseg / 4 + 1024));
+    if (resident_halo_bytes((int)cap) > H->halo_room) cap = nseg;
+    if (resident_halo_bytes((int)cap) > H->halo_room) return LBM_OK;
     H->halo_cap = 0;  // a growth that fails has freed the buffer
-    CU(H->halo.reserve(resident_halo_bytes((int)std::max(nseg, cap))));
+    H->halo.release();
+    CU(H->halo.reserve(resident_halo_bytes((int)cap)));
     CU(cudaMemsetAsync(H->halo.p, 0, H->halo.cap, E->stream));  // no tag in it may match a future one
     H->halo_epoch = 1;
-    H->halo_cap = (int)std::max(nseg, cap);
+    H->halo_cap = (int)cap;
   }
   *ok = true;
   return LBM_OK;

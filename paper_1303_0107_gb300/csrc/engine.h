@@ -128,6 +128,7 @@ struct Engine {
   GrowBuf halo;
   ResidentShape rshape{};
   int halo_cap = 0;        // segments the halo buffer holds
+  size_t halo_room = SIZE_MAX;  // bytes it may take (the request loop's budget leaves it so much)
   unsigned halo_epoch = 1;
 
   // compacted fluid-cell tasks (step.persistent == 3): the list and the
@@ -188,6 +189,9 @@ lbm_status rebuild_worklist(Engine* E);
 // Shape and halo buffer of a resident launch over the current work-list;
 // *ok: the set fits the chip.
 lbm_status resident_prepare(Engine* E, bool* ok, int max_own);
+// Bytes the halo buffer may take from here on; a larger one is freed (the
+// stream is idle).
+void set_halo_room(Engine* E, size_t bytes);
 // Whether the next n_steps of E step on the chip by rule (E->resident_now).
 lbm_status choose_resident(Engine* E, int64_t n_steps);
 // Take the work-list's length copied by the last rebuild (the stream has been

@@ -170,6 +170,7 @@ void lbm_server_s::loop() {
   bool changed = false;
   for (;;) {
     std::vector<Pending> adm;
+    int64_t charged = 0;
     {
       std::unique_lock<std::mutex> lk(mu);
       cv_work.wait(lk, [&] { return stop || !queue.empty() || !slots.empty(); });
@@ -187,7 +188,11 @@ void lbm_server_s::loop() {
       st.queued = (int32_t)queue.size();
       st.resident_bytes = resident;
       st.peak_resident_bytes = std::max(st.peak_resident_bytes, resident);
+      charged = resident;
     }
+    // the halo words of the on-chip steps are in no request's charge: they take
+    // what the budget has left, else the tick steps per phase
+    set_halo_room(E, (size_t)std::max<int64_t>(0, budget - charged));
     NvtxRange nvtx("lbm_server_tick");  // admission, exchange, steps, retirement
     const double t_tick = now();
     for (Pending& p : adm) {
