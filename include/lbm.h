@@ -300,6 +300,11 @@ void lbm_debug_fail_alloc(int64_t after);
  * lbm_load_state restores a state).  No device fault is involved.         */
 void lbm_debug_barrier_timeout(int32_t on);
 
+/* 1 if the bytes lie in one allocation in the current device's memory: states
+ * and fields are copied by a kernel to and from such buffers, by the CUDA
+ * runtime, with its own checks, otherwise.  Nothing is accessed.            */
+int32_t lbm_debug_on_device(const void* p, size_t bytes);
+
 /* Test hook of the bounds-checked build (built with -DLBM_CHECK_BOUNDS, loaded
  * with LBM_CHECKED=1 by the Python binding): that build surrounds every
  * lattice's population planes with canary blocks and checks them after each

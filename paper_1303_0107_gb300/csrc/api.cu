@@ -51,6 +51,7 @@ void lbm_transfer_bytes(uint64_t* h2d, uint64_t* d2h) { transfer_bytes(h2d, d2h)
 
 void lbm_debug_fail_alloc(int64_t after) { set_alloc_failure(after); }
 
+int32_t lbm_debug_on_device(const void* p, size_t bytes) { return on_this_device(p, bytes) ? 1 : 0; }
 void lbm_debug_barrier_timeout(int32_t on) { set_barrier_timeout_test(on); }
 
 lbm_status lbm_debug_damage_canary(lbm_handle h) {

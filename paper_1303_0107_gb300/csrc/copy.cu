@@ -39,7 +39,7 @@ template <class V>
 cudaError_t copy_as(const PlaneCopy& c, cudaStream_t stream) {
   const long long chunks = ((long long)(c.width / sizeof(V)) + 32 * kUnroll - 1) / (32 * kUnroll);
   const long long tasks = chunks * c.rows * c.planes;
-  if (tasks >= 1ll << 31) return cudaErrorInvalidValue;
+  if (tasks >= 1ll << 30) return cudaErrorInvalidValue;
   const long long blocks = (tasks + 7) / 8;
   k_copy_planes<V><<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, stream>>>(c, (int)chunks, (int)tasks);
   count_launches(1);

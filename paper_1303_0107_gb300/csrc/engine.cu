@@ -64,22 +64,39 @@ cudaError_t xfer2d(void* dst, size_t dpitch, const void* src, size_t spitch, siz
   return e;
 }
 
-namespace {
-bool on_this_device(const void* p) {
+bool on_this_device(const void* p, size_t bytes) {
+  using Range = int (*)(unsigned long long*, size_t*, unsigned long long);  // cuMemGetAddressRange
+  static const Range range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r{};
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Range>(f);
+  }();
   cudaPointerAttributes a{};
   int dev = -1;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+  if (!range || cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev;
+  unsigned long long base = 0;
+  size_t size = 0;
+  return a.type == cudaMemoryTypeDevice && a.device == dev && range(&base, &size, (uintptr_t)p) == 0 &&
+         bytes <= size && (uintptr_t)p - base <= size - bytes;
 }
-}  // namespace
 
 cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream) {
-  // (a launch takes fewer than 2^31 pieces of at least 128 bytes)
-  const bool fits = (c.width / 128 + 1) * (size_t)c.rows * (size_t)c.planes < (size_t)1 << 31;
-  if (fits && on_this_device(c.dst) && on_this_device(c.src)) return launch_copy_planes(c, stream);
+  // (a launch takes fewer than 2^30 pieces of at least 128 bytes)
+  const bool fits = (c.width / 128 + 1) * (size_t)c.rows * (size_t)c.planes < (size_t)1 << 30;
+  auto extent = [&](size_t plane, size_t pitch) {
+    return (size_t)(c.planes - 1) * plane + (size_t)(c.rows - 1) * pitch + c.width;
+  };
+  if (fits && on_this_device(c.dst, extent(c.dst_plane, c.dst_pitch)) &&
+      on_this_device(c.src, extent(c.src_plane, c.src_pitch)))
+    return launch_copy_planes(c, stream);
   for (int k = 0; k < c.planes; ++k) {
     const cudaError_t e = xfer2d(static_cast<char*>(c.dst) + k * c.dst_plane, c.dst_pitch,
                                  static_cast<const char*>(c.src) + k * c.src_plane, c.src_pitch, c.width,
@@ -1923,7 +1940,7 @@ lbm_status engine_read(Engine* E, int i, uint32_t which, void* dst, size_t dst_b
   switch (which) {
     case LBM_FIELD_MASK:
       if (dst_bytes < ncell) return fail(LBM_ERR_ARG, "dst too small");
-      if (on_this_device(dst)) {
+      if (on_this_device(dst, ncell)) {
         CU(launch_unpack_mask(m->mask, m->nx, m->ny, m->wpr, static_cast<uint8_t*>(dst), E->stream));
         break;
       }

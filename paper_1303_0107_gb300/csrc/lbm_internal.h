@@ -303,8 +303,11 @@ struct FillEntry {
 };
 // list: device; largest: bytes of its largest entry
 cudaError_t launch_fill_list(const FillEntry* list, int n, size_t largest, int sm_count, cudaStream_t stream);
-// A PlaneCopy by the kernel where both sides are device memory of the current
-// device, else by the runtime as a copy of that kind.
+// Whether the bytes lie in one allocation in the current device's memory: a
+// kernel may then access them (a runtime copy checks that by itself).
+bool on_this_device(const void* p, size_t bytes);
+// A PlaneCopy by the kernel where both sides are such memory, else by the
+// runtime as a copy of that kind.
 cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream);
 
 // ---- geometry / work-list (worklist.cu) ------------------------------------

@@ -176,6 +176,8 @@ def load_library(path=None):
     L.lbm_server_cancel.argtypes = [S, ctypes.c_int64]
     L.lbm_debug_fail_alloc.argtypes = [ctypes.c_int64]
     L.lbm_debug_fail_alloc.restype = None
+    L.lbm_debug_on_device.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
+    L.lbm_debug_on_device.restype = ctypes.c_int32
     L.lbm_debug_barrier_timeout.argtypes = [ctypes.c_int32]
     L.lbm_debug_barrier_timeout.restype = None
     L.lbm_debug_damage_canary.argtypes = [H]
