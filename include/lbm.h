@@ -357,11 +357,17 @@ lbm_status lbm_kernel_time(lbm_handle h, int reset, double* ms, int64_t* launche
  * updates at once (1 or 2), and stages = 0 (populations loaded straight into
  * registers) or 2 / 3 (copied into shared memory that many segments ahead of
  * their update).  Unless set with lbm_set_step_config, lattices and batches
- * that fit on the device run resident solves (mode 2, reported for plain
- * lattices with two cells per thread and half a block's segments as warps;
- * the kernel also serves the symmetry plane and the other collision models
- * then) from 8 steps on, and others tune the shape on their own lattice at
- * the first solve of 256 steps or more.  Any output pointer may be NULL.  */
+ * that fit on the device run resident solves from 8 steps on (the kernel also
+ * serves the symmetry plane and the other collision models then), large plain
+ * FP32 lattices solves of 16 steps or more in sweeps (four steps in one pass
+ * over memory), and others tune the shape on their own lattice at the first
+ * solve of 256 steps or more.  Resident solves are reported as mode 2 for plain
+ * lattices, with two cells per thread and half a block's segments as warps, a
+ * shape that lbm_set_step_config accepts.  For batches, groups and lattices
+ * with a plane or a model, and for lattices in sweeps, the shape reported is
+ * that of the launches around them (short solves, leftover steps): it does not
+ * say that the chip or the sweeps are left out.  Any output pointer may be
+ * NULL.                                                                    */
 lbm_status lbm_step_config(lbm_handle h, int32_t* warps_per_block, int32_t* grid, int32_t* persistent,
                            int32_t* cells_per_thread, int32_t* stages);
 /* Fix the launch shape (and skip tuning): warps_per_block 4, 8, 12, 16 or

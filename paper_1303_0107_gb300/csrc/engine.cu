@@ -1496,7 +1496,7 @@ lbm_status enqueue_steps(Engine* E, int64_t n_steps, bool with_res) {
   lbm_status st;
   bool resident = E->resident_now;
   if (E->step.persistent == 2 && !debug_sync()) {
-    if ((st = resident_prepare(E, &resident, kResidentMaxOwn)) != LBM_OK) return st;
+    if ((st = resident_prepare(E, &resident, kResidentManyOwn)) != LBM_OK) return st;
     if (!resident) E->step = shape(E, kStepWarps, kDefaultGridScale);  // the list outgrew the chip
   }
   if (resident && with_res && K > kMaxResidentSteps) {  // step T - K would not lie in the last launch
@@ -2000,7 +2000,7 @@ lbm_status engine_set_step_config(Engine* E, int32_t warps_per_block, int32_t pe
   E->groups.clear();
   if (persistent == 2) {  // on-chip resident steps: the shape follows from the work-list
     bool ok = false;
-    lbm_status st = E->features ? LBM_OK : resident_prepare(E, &ok, kResidentMaxOwn);
+    lbm_status st = E->features ? LBM_OK : resident_prepare(E, &ok, kResidentManyOwn);
     if (st != LBM_OK) return st;
     if (!ok)
       return fail(LBM_ERR_ARG, "resident steps need plain BGK lattices whose segments fit in shared memory");
