@@ -1107,7 +1107,7 @@ lbm_status rebuild_worklist(Engine* E) {
   CU(launch_count_fluid(static_cast<const LatticeView*>(E->L.views.p), static_cast<const int*>(E->L.word_off.p),
                         E->n(), E->L.total_words, static_cast<unsigned long long*>(E->fluid_dev.p), E->stream));
   if (!E->in_group || E->resident_parent) {
-    CU(cudaMemcpyAsync(E->h_nseg, E->n_segs.p, sizeof(int), cudaMemcpyDeviceToHost, E->stream));
+    CU(xfer(E->h_nseg, E->n_segs.p, sizeof(int), cudaMemcpyDeviceToHost, E->stream));
     E->nseg_copied = true;
   }
   DEBUG_SYNC(E, "work-list");
@@ -1281,7 +1281,7 @@ lbm_status members_reset(Engine* E) {
     cudaGetLastError();
     return each_member_reset(E);
   }
-  CU(cudaMemcpyAsync(E->fill_list.p, list.data(), sizeof(FillEntry) * list.size(), cudaMemcpyHostToDevice, E->stream));
+  CU(xfer(E->fill_list.p, list.data(), sizeof(FillEntry) * list.size(), cudaMemcpyHostToDevice, E->stream));
   constexpr int kMost = 65535;  // blocks in y
   for (size_t i = 0; i < list.size(); i += kMost)
     CU(launch_fill_list(static_cast<const FillEntry*>(E->fill_list.p) + i, (int)std::min<size_t>(kMost, list.size() - i),
@@ -1391,8 +1391,8 @@ bool group_bytes_set() { return std::getenv("LBM_GROUP_BYTES") != nullptr; }
 lbm_status resident_parts(Engine* E, std::vector<std::vector<Member*>>* parts) {
   const int n = E->n(), total = E->L.total_seg_words;
   std::vector<int> offs(total + 1);  // list index of every segment word
-  CU(cudaMemcpyAsync(offs.data(), static_cast<const int*>(E->seg_scratch.p) + total, sizeof(int) * (total + 1),
-                     cudaMemcpyDeviceToHost, E->stream));
+  CU(xfer(offs.data(), static_cast<const int*>(E->seg_scratch.p) + total, sizeof(int) * (total + 1),
+          cudaMemcpyDeviceToHost, E->stream));
   CU(cudaStreamSynchronize(E->stream));
   std::vector<int> count(n), order(n);
   for (int i = 0; i < n; ++i) {
@@ -1642,8 +1642,8 @@ lbm_status choose_sweep(Engine* E, int64_t n_steps) {
     CU(launch_build_sweep(E->L.h_views[0], list, E->stream));
     int cost = 0;
     unsigned long long fluid = 0;
-    CU(cudaMemcpyAsync(&cost, list.total_cost, sizeof(cost), cudaMemcpyDeviceToHost, E->stream));
-    CU(cudaMemcpyAsync(&fluid, E->fluid_dev.p, sizeof(fluid), cudaMemcpyDeviceToHost, E->stream));
+    CU(xfer(&cost, list.total_cost, sizeof(cost), cudaMemcpyDeviceToHost, E->stream));
+    CU(xfer(&fluid, E->fluid_dev.p, sizeof(fluid), cudaMemcpyDeviceToHost, E->stream));
     CU(cudaStreamSynchronize(E->stream));
     E->sweep_pays = fluid * cell_bytes > (size_t)E->l2_bytes && (unsigned long long)cost * 10 <= fluid;
     E->sweep_valid = true;
