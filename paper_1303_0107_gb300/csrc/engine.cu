@@ -1222,6 +1222,8 @@ lbm_status engine_set_members(Engine* E, const std::vector<Member*>& members) {
     E->step.persistent = 0;
   }
   E->m = members;
+  E->sweep_no = E->sweep_no_start = 0;
+  E->exchanged = false;
   const size_t n = members.size();
   lbm_status st = layout_build(E->L, E->m, E->stream);
   if (st != LBM_OK) return st;
@@ -1293,6 +1295,8 @@ lbm_status members_reset(Engine* E) {
 lbm_status engine_reset(Engine* E) {
   lbm_status st = E->n() == 1 ? each_member_reset(E) : members_reset(E);
   if (st != LBM_OK) return st;
+  E->sweep_no = E->sweep_no_start;
+  E->exchanged = false;
   st = rebuild_worklist(E);
   if (st != LBM_OK) return st;
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long) * E->n(), cudaMemcpyDeviceToHost,
@@ -1628,9 +1632,16 @@ lbm_status choose_sweep(Engine* E, int64_t n_steps) {
     return LBM_OK;
   const Member* m = E->m[0];
   const size_t cell_bytes = 9 * sizeof(float), bytes = cell_bytes * m->plane, rows = (size_t)sweep_rows(m->nx, m->ny);
-  if (!forced && bytes <= (size_t)E->l2_bytes) return LBM_OK;
+  // (an exchange keeps the number of fluid cells)
+  if (!forced && ((size_t)m->fluid_cells * cell_bytes <= (size_t)E->l2_bytes || E->sweep_no > 0)) return LBM_OK;
   if (m->ny >= 1 << kSweepRowBits || rows / m->ny > (size_t)1 << (31 - kSweepRowBits) || rows >= (size_t)1 << 26)
     return LBM_OK;  // more than a list entry and the sums hold
+  if (E->second.cap < bytes) {
+    // a second buffer only out of plenty: what else the program allocates fits as before
+    size_t free_bytes = 0, all = 0;
+    CU(cudaMemGetInfo(&free_bytes, &all));
+    if (bytes > free_bytes / 8) return LBM_OK;
+  }
   if (!E->sweep_valid) {
     cudaError_t e = E->sweep_buf.reserve(sweep_list(m->nx, m->ny, nullptr).ints * sizeof(int));
     if (e == cudaErrorMemoryAllocation) {  // the per-phase kernels need none of this
@@ -1645,15 +1656,15 @@ lbm_status choose_sweep(Engine* E, int64_t n_steps) {
     CU(xfer(&cost, list.total_cost, sizeof(cost), cudaMemcpyDeviceToHost, E->stream));
     CU(xfer(&fluid, E->fluid_dev.p, sizeof(fluid), cudaMemcpyDeviceToHost, E->stream));
     CU(cudaStreamSynchronize(E->stream));
-    E->sweep_pays = fluid * cell_bytes > (size_t)E->l2_bytes && (unsigned long long)cost * 10 <= fluid;
+    const long long over = 10 * (long long)cost - (long long)fluid;
+    E->sweep_pays = fluid * cell_bytes > (size_t)E->l2_bytes && over <= 0;
     E->sweep_valid = true;
+    // each cell moved is a fluid and a solid one
+    E->sweep_no = over > 0 ? (over - 1) / (10 * 2 * kSweepCostPerCell) + 1 : 0;
+    if (!E->exchanged) E->sweep_no_start = E->sweep_no;
   }
   if (!E->sweep_pays && !forced) return LBM_OK;
   if (E->second.cap < bytes) {
-    // a second buffer only out of plenty: what else the program allocates fits as before
-    size_t free_bytes = 0, all = 0;
-    CU(cudaMemGetInfo(&free_bytes, &all));
-    if (bytes > free_bytes / 8) return LBM_OK;
     cudaError_t e = E->second.reserve(bytes);
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
@@ -1720,6 +1731,8 @@ lbm_status enqueue_exchange(Engine* E, const std::vector<int>& which, const int3
     Member* m = E->m[i];
     if (m->p.reinit == LBM_REINIT_COLD) CU(cudaMemsetAsync(m->f, 0, 9 * m->plane * sb, E->stream));
   }
+  E->exchanged = true;
+  for (int k = 0; k < nx_; ++k) E->sweep_no -= n_swap[k];
   for (int k = 0; k < nx_; ++k) E->seg_bound += n_swap[k];  // a new fluid cell opens at most one segment
   E->seg_bound = std::min<long long>(E->seg_bound, E->L.total_seg_words);
   for (Engine* g : E->groups) {
@@ -1871,6 +1884,8 @@ lbm_status restore_state(Engine* E, Member* m) {
   CU(xfer(m->f, b, z.f, cudaMemcpyDeviceToDevice, E->stream));
   CU(xfer(m->mask_base, b + z.f, z.mask, cudaMemcpyDeviceToDevice, E->stream));
   CU(xfer(m->drho, b + z.f + z.mask, z.fields, cudaMemcpyDeviceToDevice, E->stream));
+  E->sweep_no = 0;  // (the mask of some earlier design)
+  E->exchanged = true;
   lbm_status st = rebuild_worklist(E);
   if (st != LBM_OK) return st;
   CU(xfer(E->h_count, E->fluid_dev.p, sizeof(unsigned long long), cudaMemcpyDeviceToHost, E->stream));

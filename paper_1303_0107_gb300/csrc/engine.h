@@ -148,6 +148,10 @@ struct Engine {
   GrowBuf sweep_buf, second;
   bool sweep_valid = false;
   bool sweep_pays = false;  // the rule's answer for the list
+  // > 0: the rule says no, and so it will until exchanges have moved that many
+  // cells each way; the value at the creation state, to which a reset returns
+  long long sweep_no = 0, sweep_no_start = 0;
+  bool exchanged = false;   // the masks are not those of the creation state
   bool sweep_now = false;   // the solve being enqueued steps in sweeps
 
   cudaGraphExec_t graphs[4] = {nullptr, nullptr, nullptr, nullptr};  // 512, 64, 8 and 1 pairs

@@ -245,6 +245,9 @@ cudaError_t launch_stream_collide_resident(int precision, int features, const La
 // of the lattice's layout; G's solid cells are left alone).
 constexpr int kSweepSteps = 4;
 constexpr int kSweepBlocks = 2;    // blocks per SM
+// An exchanged cell changes the cost of at most three rows of two tiles, by at
+// most the largest cost of a row (sweep.cu).
+constexpr int kSweepMaxCost = 18, kSweepCostPerCell = 6 * kSweepMaxCost;
 constexpr int kSweepRowBits = 19;  // list entry: tile << 19 | row
 long long sweep_rows(int nx, int ny);  // rows of all tiles
 // The rows of all tiles that hold fluid, with their costs, and what builds

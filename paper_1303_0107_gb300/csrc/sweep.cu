@@ -55,7 +55,7 @@ constexpr int kRow = 9 * kCols;            // values of a row
 constexpr int kPad = 32;                   // words before the first ring (a window's lane 0 reads one to the left)
 constexpr unsigned kSpinLimit = 1u << 22;
 // relative time of a turn on a row: all windows open, one with a wall, one with a port
-constexpr int kCostOpen = 8, kCostClosed = 12, kCostPort = 18;
+constexpr int kCostOpen = 8, kCostClosed = 12, kCostPort = kSweepMaxCost;
 
 constexpr int kHalo = kSteps, kOut = kCols - 2 * kHalo;
 constexpr int kSmem = 4 * (kPad + kRing0 * kRow + (kSteps - 1) * kRing * kRow + kPad);
