@@ -42,3 +42,33 @@ def test_no_row_list_where_the_answer_stays_no(monkeypatch):
     b.close()
     assert got[0] > want[0]  # the first question is asked
     assert got[1:] == want[1:]
+
+
+FIELDS = (L.FIELD_MASK, L.FIELD_DRHO, L.FIELD_UX, L.FIELD_UY, L.FIELD_POPS)
+
+
+@pytest.mark.parametrize("fails", [-1, 0, 1])  # no allocation; the row list's; the second buffer's
+def test_the_rule_takes_sweeps_beyond_the_cache(fails):
+    cells = I.channel_array(4000, 2000, 4)  # 144 MB of fluid populations in open rows
+    a, b = (L.Lattice(cells, 0.6, 0.05, residual_every=20) for _ in range(2))
+    b.set_step_config(8, persistent=False)
+    for i, step in enumerate((lambda h: h.solve(8), lambda h: h.solve(100), lambda h: h.optimize_step(200, 40),
+                              lambda h: h.solve(8), lambda h: h.solve(50))):
+        if i == 1:
+            L.lib.debug_fail_alloc(fails)
+        n0 = L.kernel_launches()
+        ra = step(a)
+        n1 = L.kernel_launches()
+        L.lib.debug_fail_alloc(-1)
+        rb = step(b)
+        per_phase = L.kernel_launches() - n1
+        if i in (0, 3) or (i == 1 and fails >= 0):  # short, or no memory: one launch per phase
+            assert n1 - n0 >= per_phase, i
+        else:
+            assert n1 - n0 < per_phase, i
+        assert ra["dp"] == rb["dp"] and ra["m_in"] == rb["m_in"] and ra["residual"] == rb["residual"], i
+        assert list(ra["m_out"]) == list(rb["m_out"])
+        for f in FIELDS:
+            assert np.array_equal(a.read(f), b.read(f)), (i, f)
+    a.close()
+    b.close()
