@@ -402,9 +402,12 @@ void set_last_error(const std::string& msg);
 bool debug_sync();
 
 #ifdef LBM_CHECK_BOUNDS
-// Bounds-checked builds: every global access of the step and reduction
-// kernels is checked against its allocation; a violation is printed and the
-// access skipped.
+// Bounds-checked builds: every population and field access of the step,
+// resident, sweep, exchange and reduction kernels is checked against its
+// allocation (the copies of a sweep's input by its tensor map), and of the
+// resident kernels the shared-memory and halo words that their tables name; a
+// violation is printed and the access skipped.  The copy kernels' ranges are
+// checked on the host, in every build (copy_planes).
 __device__ __forceinline__ bool lbm_in_bounds(long long i, long long n, int line) {
   if (i >= 0 && i < n) return true;
   printf("lbm bounds: line %d index %lld extent %lld block %d thread %d\n", line, i, n, blockIdx.x,

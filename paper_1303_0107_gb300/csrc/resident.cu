@@ -284,6 +284,7 @@ __device__ __forceinline__ void ports_of(float (&g)[9], unsigned slot_flags, con
 __device__ __forceinline__ void write_moments(const SlotInfo& si, int lane, bool last, float drho, float ux, float uy) {
   const LatticeView& L = *si.L;
   const long long c = si.row + lane;
+  if (!LBM_OK_IDX(c, L.plane)) return;
   L.drho[c] = drho;
   (last ? L.ux : L.ux_prev)[c] = ux;
   (last ? L.uy : L.uy_prev)[c] = uy;
@@ -497,12 +498,14 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
           }
         }
       }
+      if (!LBM_OK_IDX(o, kZeroWord + 1)) o = kZeroWord;
       off[i - 1] = r ? off[i - 1] | (unsigned)o << 16 : (unsigned)o;
     }
     // what other blocks read of this segment, and what it reads of theirs
     bool rem[8];
 #pragma unroll
-    for (int p = 0; p < 8; ++p) rem[p] = s_nbq[t][p] >= 0 && (s_nbq[t][p] < s0 || s_nbq[t][p] >= s1);
+    for (int p = 0; p < 8; ++p)
+      rem[p] = s_nbq[t][p] >= 0 && (s_nbq[t][p] < s0 || s_nbq[t][p] >= s1) && LBM_OK_IDX(s_nbq[t][p], halo_cap);
     const bool side = rem[0] || rem[2];
     if (rem[1] || rem[4] || rem[5]) sf |= kPubUp;
     if (rem[3] || rem[6] || rem[7] || (plane && side)) sf |= kPubDown;
@@ -523,7 +526,7 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
       if (plane && rem[0]) pi.edge[8 * r + 5] = word(0, kUnitDown, 0, 1);
       pi.rho0[r] = L.rho0;
       pi.omega[r] = L.omega;
-      pi.unit0[r] = q * 3 * kUnitWords;
+      pi.unit0[r] = LBM_OK_IDX(q, halo_cap) ? q * 3 * kUnitWords : 0;
       const int ol = L.nx - 1 - (w << 5);
       s_slots[j] = SlotInfo{w == 0 && !(mc & 1u) ? 0 : -1, ol < 32 && !((mc >> (ol & 31)) & 1u) ? ol : -1,
                             w == 0 ? L.u_in[y] : 0.0f, L.port_scheme == LBM_PORTS_ZOU_HE,
@@ -536,30 +539,31 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
     // own populations and the ghost words of step 0 from the canonical layout
     const T* F = static_cast<const T*>(L.f);
     const int pl = (int)L.plane, cell = y * L.pitch + x;
+    auto from = [&](int at) { return LBM_OK_IDX(at, L.f_elems) ? P::ld(F + at) : 0.0f; };
 #pragma unroll
-    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = P::ld(F + i * pl + cell);
+    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = from(i * pl + cell);
     float* gw = buf0 + gbase;
     if (rem[1]) {
-      gw[1 + lane] = P::ld(F + 4 * pl + cell + L.pitch);
-      gw[kGhostRow + 1 + lane] = P::ld(F + 7 * pl + cell + L.pitch);
-      gw[2 * kGhostRow + 1 + lane] = P::ld(F + 8 * pl + cell + L.pitch);
+      gw[1 + lane] = from(4 * pl + cell + L.pitch);
+      gw[kGhostRow + 1 + lane] = from(7 * pl + cell + L.pitch);
+      gw[2 * kGhostRow + 1 + lane] = from(8 * pl + cell + L.pitch);
     }
     if (rem[3]) {
-      gw[3 * kGhostRow + 1 + lane] = P::ld(F + 2 * pl + cell - L.pitch);
-      gw[4 * kGhostRow + 1 + lane] = P::ld(F + 5 * pl + cell - L.pitch);
-      gw[5 * kGhostRow + 1 + lane] = P::ld(F + 6 * pl + cell - L.pitch);
+      gw[3 * kGhostRow + 1 + lane] = from(2 * pl + cell - L.pitch);
+      gw[4 * kGhostRow + 1 + lane] = from(5 * pl + cell - L.pitch);
+      gw[5 * kGhostRow + 1 + lane] = from(6 * pl + cell - L.pitch);
     }
     if (lane == 0) {
-      if (rem[2]) gw[kGhostWest] = P::ld(F + 1 * pl + cell - 1);
-      if (rem[5]) gw[2 * kGhostRow] = P::ld(F + 8 * pl + cell + L.pitch - 1);
-      if (rem[6]) gw[4 * kGhostRow] = P::ld(F + 5 * pl + cell - L.pitch - 1);
-      if (plane && rem[2]) gw[4 * kGhostRow] = P::ld(F + 8 * pl + cell - 1);
+      if (rem[2]) gw[kGhostWest] = from(1 * pl + cell - 1);
+      if (rem[5]) gw[2 * kGhostRow] = from(8 * pl + cell + L.pitch - 1);
+      if (rem[6]) gw[4 * kGhostRow] = from(5 * pl + cell - L.pitch - 1);
+      if (plane && rem[2]) gw[4 * kGhostRow] = from(8 * pl + cell - 1);
     }
     if (lane == 31) {
-      if (rem[0]) gw[kGhostEast] = P::ld(F + 3 * pl + cell + 1);
-      if (rem[4]) gw[kGhostRow + 33] = P::ld(F + 7 * pl + cell + L.pitch + 1);
-      if (rem[7]) gw[5 * kGhostRow + 33] = P::ld(F + 6 * pl + cell - L.pitch + 1);
-      if (plane && rem[0]) gw[5 * kGhostRow + 33] = P::ld(F + 7 * pl + cell + 1);
+      if (rem[0]) gw[kGhostEast] = from(3 * pl + cell + 1);
+      if (rem[4]) gw[kGhostRow + 33] = from(7 * pl + cell + L.pitch + 1);
+      if (rem[7]) gw[5 * kGhostRow + 33] = from(6 * pl + cell - L.pitch + 1);
+      if (plane && rem[0]) gw[5 * kGhostRow + 33] = from(7 * pl + cell + 1);
     }
   }
   const SlotInfo* si = s_slots + S * warp;
@@ -596,7 +600,8 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
     T* F = static_cast<T*>(L.f) + si[r].row + lane;
     const int pl = (int)L.plane;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) P::st(F + i * pl, sm[own + r * kSegWords + i * 32]);
+    for (int i = 0; i < 9; ++i)
+      if (LBM_OK_IDX(si[r].row + lane + i * pl, L.f_elems)) P::st(F + i * pl, sm[own + r * kSegWords + i * 32]);
   }
 }
 
@@ -891,12 +896,13 @@ __global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
             }
           }
         }
+        if (!LBM_OK_IDX(o, 2 * kManyPairs * kSegWords + 32)) o = outside;
         off[i - 1] |= (unsigned)o << (16 * r);
       }
       // what other blocks read of this segment, and what it reads of theirs
       bool rem[8];
 #pragma unroll
-      for (int d = 0; d < 8; ++d) rem[d] = is_remote(s_nbq[t][d]);
+      for (int d = 0; d < 8; ++d) rem[d] = is_remote(s_nbq[t][d]) && LBM_OK_IDX(s_nbq[t][d], halo_cap);
       const bool side = rem[0] || rem[2];
       unsigned sf = 0;
       if (rem[1] || rem[4] || rem[5]) sf |= kPubUp;
@@ -918,7 +924,7 @@ __global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
         if (plane && rem[0]) pi.edge[8 * r + 5] = word(0, kUnitDown, 0, 1);
         pi.rho0[r] = L.rho0;
         pi.omega[r] = L.omega;
-        pi.unit0[r] = q * 3 * kUnitWords;
+        pi.unit0[r] = LBM_OK_IDX(q, halo_cap) ? q * 3 * kUnitWords : 0;
         const int ol = L.nx - 1 - (w << 5);
         m.slots[j] = SlotInfo{w == 0 && !(mc & 1u) ? 0 : -1, ol < 32 && !((mc >> (ol & 31)) & 1u) ? ol : -1,
                               w == 0 ? L.u_in[y] : 0.0f, L.port_scheme == LBM_PORTS_ZOU_HE,
@@ -947,7 +953,9 @@ __global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
       float g[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
-        g[i] = (si.fluid >> lane) & 1u ? P::ld(F + (long long)i * pl) : 0.0f;
+        g[i] = (si.fluid >> lane) & 1u && LBM_OK_IDX(si.row + lane + (long long)i * pl, si.L->f_elems)
+                   ? P::ld(F + (long long)i * pl)
+                   : 0.0f;
         m.rows[2 * p + r][i * 32 + lane] = g[i];
       }
       if (sf & kPublishes) publish(halo + parity + m.pairs[p].unit0[r] + lane, sf, lane, g, epoch0);
@@ -982,7 +990,9 @@ __global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
     T* F = static_cast<T*>(si.L->f) + si.row + lane;
     const int pl = (int)si.L->plane;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) P::st(F + (long long)i * pl, m.rows[j][i * 32 + lane]);
+    for (int i = 0; i < 9; ++i)
+      if (LBM_OK_IDX(si.row + lane + (long long)i * pl, si.L->f_elems))
+        P::st(F + (long long)i * pl, m.rows[j][i * 32 + lane]);
   }
 }
 

@@ -178,8 +178,10 @@ __device__ __forceinline__ void window_step(const LatticeView& L, const float* i
       out[i * kCols + 32] = b;
     }
   } else {
-    float* f = G + ((long long)y * L.pitch + x);
-    const bool wa = fa && x >= x_lo && x < x_hi, wb = fb && x + 32 >= x_lo && x + 32 < x_hi;
+    const long long c = (long long)y * L.pitch + x;
+    float* f = G + c;
+    const bool wa = fa && x >= x_lo && x < x_hi && LBM_OK_IDX(c, L.plane),
+               wb = fb && x + 32 >= x_lo && x + 32 < x_hi && LBM_OK_IDX(c + 32, L.plane);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       float a, b;
