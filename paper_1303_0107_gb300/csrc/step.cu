@@ -91,7 +91,7 @@ __device__ __forceinline__ void seg_prologue(const LatticeView* __restrict__ vie
   const int y = sr.yw >> kSegWordBits;
   const int w = sr.yw & ((1 << kSegWordBits) - 1);
 #ifdef LBM_CHECK_BOUNDS
-  if (valid && (sr.lattice < 0 || y < 1 || y > L->ny - 2 || w < 0 || w >= L->wpr)) {
+  if (valid && (sr.lattice < 0 || y < first_step_row(*L) || y > L->ny - 2 || w < 0 || w >= L->wpr)) {
     if (lane == 0) printf("lbm bounds: bad segment: lattice %d y %d w %d\n", sr.lattice, y, w);
     valid = false;
     L = views;

@@ -54,3 +54,4 @@ def test_no_access_outside():
     want = _run()
     assert len(want) == 20
     assert _run(LBM_CHECKED="1")[:15] == want[:15]
+    assert _run(LBM_CHECKED="1", LBM_RESIDENT="0", LBM_SWEEP="1")[:15] == want[:15]  # sweeps, and per phase
