@@ -2,6 +2,8 @@
 // exchange and read-back.  Host code only: it validates arguments, owns
 // device memory and enqueues the kernels of step.cu, worklist.cu, reduce.cu
 // and oc.cu on the engine's stream.
+#include <cuda.h>  // pointer attributes (types only: the call is looked up at run time)
+
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -65,27 +67,34 @@ cudaError_t xfer2d(void* dst, size_t dpitch, const void* src, size_t spitch, siz
 }
 
 bool on_this_device(const void* p, size_t bytes) {
-  using Range = int (*)(unsigned long long*, size_t*, unsigned long long);  // cuMemGetAddressRange
-  static const Range range = [] {
+  // one driver call for type, device and range (a pointer it does not know has none)
+  using Attributes = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Attributes attributes = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult r{};
-    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
         r != cudaDriverEntryPointSuccess) {
       cudaGetLastError();
       f = nullptr;
     }
-    return reinterpret_cast<Range>(f);
+    return reinterpret_cast<Attributes>(f);
   }();
-  cudaPointerAttributes a{};
-  int dev = -1;
-  if (!range || cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  CUmemorytype type{};
+  unsigned managed = 0;
+  int on = -1, dev = -2;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  void* data[] = {&type, &managed, &on, &base, &size};
+  if (!attributes || attributes(5, what, data, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS ||
+      cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  unsigned long long base = 0;
-  size_t size = 0;
-  return a.type == cudaMemoryTypeDevice && a.device == dev && range(&base, &size, (uintptr_t)p) == 0 &&
-         bytes <= size && (uintptr_t)p - base <= size - bytes;
+  return type == CU_MEMORYTYPE_DEVICE && !managed && on == dev && bytes <= size &&
+         (uintptr_t)p - base <= size - bytes;
 }
 
 cudaError_t copy_planes(const PlaneCopy& c, cudaMemcpyKind kind, cudaStream_t stream) {

@@ -539,32 +539,33 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
     // own populations and the ghost words of step 0 from the canonical layout
     const T* F = static_cast<const T*>(L.f);
     const int pl = (int)L.plane, cell = y * L.pitch + x;
-    auto from = [&](int at) { return LBM_OK_IDX(at, L.f_elems) ? P::ld(F + at) : 0.0f; };
+#define FROM(at) (LBM_OK_IDX((at), L.f_elems) ? P::ld(F + at) : 0.0f)
 #pragma unroll
-    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = from(i * pl + cell);
+    for (int i = 0; i < 9; ++i) buf0[base + i * 32 + lane] = FROM(i * pl + cell);
     float* gw = buf0 + gbase;
     if (rem[1]) {
-      gw[1 + lane] = from(4 * pl + cell + L.pitch);
-      gw[kGhostRow + 1 + lane] = from(7 * pl + cell + L.pitch);
-      gw[2 * kGhostRow + 1 + lane] = from(8 * pl + cell + L.pitch);
+      gw[1 + lane] = FROM(4 * pl + cell + L.pitch);
+      gw[kGhostRow + 1 + lane] = FROM(7 * pl + cell + L.pitch);
+      gw[2 * kGhostRow + 1 + lane] = FROM(8 * pl + cell + L.pitch);
     }
     if (rem[3]) {
-      gw[3 * kGhostRow + 1 + lane] = from(2 * pl + cell - L.pitch);
-      gw[4 * kGhostRow + 1 + lane] = from(5 * pl + cell - L.pitch);
-      gw[5 * kGhostRow + 1 + lane] = from(6 * pl + cell - L.pitch);
+      gw[3 * kGhostRow + 1 + lane] = FROM(2 * pl + cell - L.pitch);
+      gw[4 * kGhostRow + 1 + lane] = FROM(5 * pl + cell - L.pitch);
+      gw[5 * kGhostRow + 1 + lane] = FROM(6 * pl + cell - L.pitch);
     }
     if (lane == 0) {
-      if (rem[2]) gw[kGhostWest] = from(1 * pl + cell - 1);
-      if (rem[5]) gw[2 * kGhostRow] = from(8 * pl + cell + L.pitch - 1);
-      if (rem[6]) gw[4 * kGhostRow] = from(5 * pl + cell - L.pitch - 1);
-      if (plane && rem[2]) gw[4 * kGhostRow] = from(8 * pl + cell - 1);
+      if (rem[2]) gw[kGhostWest] = FROM(1 * pl + cell - 1);
+      if (rem[5]) gw[2 * kGhostRow] = FROM(8 * pl + cell + L.pitch - 1);
+      if (rem[6]) gw[4 * kGhostRow] = FROM(5 * pl + cell - L.pitch - 1);
+      if (plane && rem[2]) gw[4 * kGhostRow] = FROM(8 * pl + cell - 1);
     }
     if (lane == 31) {
-      if (rem[0]) gw[kGhostEast] = from(3 * pl + cell + 1);
-      if (rem[4]) gw[kGhostRow + 33] = from(7 * pl + cell + L.pitch + 1);
-      if (rem[7]) gw[5 * kGhostRow + 33] = from(6 * pl + cell - L.pitch + 1);
-      if (plane && rem[0]) gw[5 * kGhostRow + 33] = from(7 * pl + cell + 1);
+      if (rem[0]) gw[kGhostEast] = FROM(3 * pl + cell + 1);
+      if (rem[4]) gw[kGhostRow + 33] = FROM(7 * pl + cell + L.pitch + 1);
+      if (rem[7]) gw[5 * kGhostRow + 33] = FROM(6 * pl + cell - L.pitch + 1);
+      if (plane && rem[0]) gw[5 * kGhostRow + 33] = FROM(7 * pl + cell + 1);
     }
+#undef FROM
   }
   const SlotInfo* si = s_slots + S * warp;
   if (lane == 0) pi.flags = flags;
