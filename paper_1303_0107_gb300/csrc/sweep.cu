@@ -308,13 +308,14 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
     int failed = 0;
     if (level > kSteps) {  // the warp that issues the copies and waits for them
       int copied = r_lo, arrived = r_lo;  // next input rows to copy and to wait for
+      int last = r_hi;                    // (after a failure none)
       auto wait_row = [&](int y) {
         const unsigned i = seq + (unsigned)(y - r_lo);
         return bar_wait(shared_addr(&s_full[i % kRing0]), (i / kRing0) & 1u) && i < give_up;
       };
       for (int k = r.k_lo - 1; k <= r.k_hi; ++k) {
         // row i takes the place of row i - 8, last read in turn i - 7
-        for (; !failed && copied <= min(k + kRing0 - 2, r_hi); ++copied) {
+        for (; copied <= min(k + kRing0 - 2, last); ++copied) {
           const unsigned slot = (seq + (unsigned)(copied - r_lo)) % kRing0;
           const unsigned bar = shared_addr(&s_full[slot]);
           if (lane == 0) {
@@ -323,7 +324,11 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, kSweepBlocks)
           }
         }
         // what the next turn reads has arrived before this one ends
-        for (; !failed && arrived <= min(k + 2, r_hi); ++arrived) failed = !wait_row(arrived);
+        for (; arrived <= min(k + 2, last); ++arrived)
+          if (!wait_row(arrived)) {
+            failed = 1;
+            last = -1;
+          }
         __syncthreads();
       }
       if (failed)  // no copy is issued after the one that failed; those in flight land (or give up) before the block leaves
