@@ -790,7 +790,8 @@ def main():
     achieved = bytes_per_launch / avg_launch_s / 1e9
     peak, peak_kind = measured_peaks()
     resident = lat.step_config()[2] == 2
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+    roofline = {"bound": "latency" if resident else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak,
                 "traffic": (profiled_traffic("resident.cu", "resident_tree_2048x1024.md",
                                              "dram_bytes_per_step_full_workload") if resident
                             else profiled_traffic("step.cu", "stream_collide_tree_2048x1024.md")),
@@ -799,7 +800,8 @@ def main():
                 "per": "time step (fluid cells x algorithmic bytes per update; mean time per step)",
                 "kernel": "k_stream_collide_resident" if resident else "k_stream_collide",
                 "note": ("populations in shared memory for the whole solve (one launch per solve), halo words in L2; "
-                         "bound by SM instruction issue" if resident else
+                         "bound by the chain of a step: frac compares with streaming the algorithmic bytes, which stay "
+                         "on the chip" if resident else
                          "lattice working set (fluid cells) is L2-resident within a solve")}
 
     # end to end through the public API, as many runs as timed steps: pinned

@@ -1,4 +1,4 @@
-// Per-cell D2Q9 arithmetic shared by the step kernels (step.cu, resident.cu):
+// Per-cell D2Q9 arithmetic shared by the step kernels (step.cu, resident.cu, sweep.cu):
 // storage conversion of the shifted populations, the moments of Eq. 2, the
 // BGK relaxation of Eq. 1 towards the second-order equilibrium of Sec. 2.1
 // (and the other collision models), and the port rules of Sec. 3.3.  Every
@@ -13,6 +13,17 @@
 
 namespace lbm {
 namespace {
+
+// D2Q9 velocities and opposites (compile-time indices after unrolling)
+__host__ __device__ constexpr int cx_of(int i) {
+  return i == 1 || i == 5 || i == 8 ? 1 : i == 3 || i == 6 || i == 7 ? -1 : 0;
+}
+__host__ __device__ constexpr int cy_of(int i) {
+  return i == 2 || i == 5 || i == 6 ? 1 : i == 4 || i == 7 || i == 8 ? -1 : 0;
+}
+__host__ __device__ constexpr int opp_of(int i) {
+  return i == 0 ? 0 : i <= 4 ? ((i + 1) & 3) + 1 : ((i - 5 + 2) & 3) + 5;
+}
 
 template <class T>
 struct Pop;

@@ -20,7 +20,7 @@
 namespace lbm {
 
 // A named range on the host timeline for profilers (NVTX: solve, time
-// steps, reductions, exchange, tuning, resident plan, server tick).  Costs
+// steps, reductions, exchange, tuning, server tick).  Costs
 // nothing measurable when no profiler is attached.
 struct NvtxRange {
   explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
@@ -116,7 +116,7 @@ struct Engine {
   int* h_bar_error = nullptr;             // pinned: grid-barrier error flag of the last solve
   bool bar_used = false;                  // the error word was cleared for the solve being enqueued, which may set it
 
-  // on-chip resident steps (step.persistent == 2): a host-side bound on the
+  // on-chip resident steps (by rule, or step.persistent == 2): a host-side bound on the
   // segments of the current work-list (exact when the list was last counted,
   // then raised by what each exchange can add), the halo buffer of tagged
   // words and the next tag

@@ -120,7 +120,8 @@ struct StepConfig {
   int stages;           // 0: populations loaded into registers; 2 or 3: staged through shared
                         //    memory that many segments ahead (one cell per thread, per-phase launches)
   int features;         // kernel build: bit 0 collision models beyond BGK, bit 1 symmetry plane
-                        //    (non-zero: one cell per thread, register loads, per-phase launches)
+                        //    (non-zero: one cell per thread, register loads, per-phase launches, or
+                        //    the resident kernels by rule)
 };
 // A fluid cell of the compacted task list: c = y * pitch + x in its lattice;
 // meta = lattice | neighbour flags (kNbE..kNbMirror) << 20 | inlet << 29 |

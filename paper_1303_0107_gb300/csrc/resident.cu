@@ -103,10 +103,6 @@ __device__ __forceinline__ int pos_of(int dy, int dw) {
   return dw < 0 ? 6 : 7;
 }
 
-// D2Q9 velocities and opposites (compile-time indices after unrolling)
-__host__ __device__ constexpr int cx_of(int i) { return i == 1 || i == 5 || i == 8 ? 1 : i == 3 || i == 6 || i == 7 ? -1 : 0; }
-__host__ __device__ constexpr int cy_of(int i) { return i == 2 || i == 5 || i == 6 ? 1 : i == 4 || i == 7 || i == 8 ? -1 : 0; }
-__host__ __device__ constexpr int opp_of(int i) { return i == 0 ? 0 : i <= 4 ? ((i + 1) & 3) + 1 : ((i - 5 + 2) & 3) + 5; }
 // ghost row of direction i arriving from above (4, 7, 8) or below (2, 5, 6)
 __host__ __device__ constexpr int ghost_row(int i) {
   return i == 4 ? 0 : i == 7 ? 1 : i == 8 ? 2 : i == 2 ? 3 : i == 5 ? 4 : 5;
@@ -592,7 +588,7 @@ __global__ void __launch_bounds__(Layout<S>::kWarps * 32, 1)
       failed = !fetch_ghosts<S>(sm + kBufWords, pi, halo, 0, epoch0 + (unsigned)k + 1u + tag_skew, lane, error);
     if (!failed) warp_step<T, FEAT, S, 1>(sm, off, own, k + 1, n_steps - 1, mom_prev, epoch0, pi, si, halo, parity, lane);
   }
-  if (__syncthreads_or(failed)) return;  // the global layout keeps the state from before the launch
+  if (__syncthreads_or(failed)) return;  // this block stores nothing; others may have ended: the state is void
   // ---- the final state (buffer 0: an even number of steps) to the canonical layout ----
 #pragma unroll
   for (int r = 0; r < S; ++r) {
@@ -983,7 +979,7 @@ __global__ void __launch_bounds__(kResidentManyWarps * 32, 1)
       if (!many_step<T, FEAT, false>(m, p, k + 1, n_steps - 1, mom_prev, epoch0, tag_skew, halo, parity, lane, error))
         n_mine = -1;
   }
-  if (__syncthreads_or(n_mine < 0)) return;  // the global layout keeps the state from before the launch
+  if (__syncthreads_or(n_mine < 0)) return;  // this block stores nothing; others may have ended: the state is void
   // ---- the final state (an even number of steps) to the canonical layout ----
   for (int j = warp; j < n_own; j += n_warps) {
     const SlotInfo& si = m.slots[j];

@@ -32,10 +32,11 @@
 // of n rows costs n + 9 turns (three more rows of the first step on either
 // side, and the pipeline of four steps two rows apart).
 //
-// What bounds it: a turn takes about 1,550 cycles, of which the collisions
-// fill the FMA pipe for 840 (two blocks a SM, so that one computes while the
-// other waits at its barrier); DRAM is idle half the time.  8192 x 4096 cells,
-// 16.8 M of them fluid, FP32: 114 us a step, per-phase kernel 193.  Three
+// What bounds it: a turn takes about 1,550 cycles, of which the FMA pipe is
+// busy for 560 (18 % of instructions counted once; a packed one holds it for
+// two cycles) and issue for 700 (two blocks a SM, so that one computes while
+// the other waits at its barrier); DRAM is idle half the time.  8192 x 4096
+// cells, 16.8 M of them fluid, FP32: 112 us a step, per-phase kernel 193.  Three
 // blocks a SM (80 registers) gave no more; a row copied as nine bulk copies by
 // nine lanes took 1,740 cycles to issue, the tensor copy one instruction.
 #include <cuda.h>  // CUtensorMap (types only: the encoder is looked up at run time)
@@ -91,10 +92,6 @@ __device__ __forceinline__ void copy_row(unsigned dst, const CUtensorMap* map, i
       "l"(map), "r"(x), "r"(y), "r"(0), "r"(bar)
       : "memory");
 }
-
-__host__ __device__ constexpr int cx_of(int i) { return i == 1 || i == 5 || i == 8 ? 1 : i == 3 || i == 6 || i == 7 ? -1 : 0; }
-__host__ __device__ constexpr int cy_of(int i) { return i == 2 || i == 5 || i == 6 ? 1 : i == 4 || i == 7 || i == 8 ? -1 : 0; }
-__host__ __device__ constexpr int opp_of(int i) { return i == 0 ? 0 : i <= 4 ? ((i + 1) & 3) + 1 : ((i - 5 + 2) & 3) + 5; }
 
 // What the windows of a tile row hold: bit w of `open` set when the cells of
 // window w and all their neighbours are fluid, of `some` when it holds a
