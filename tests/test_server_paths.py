@@ -62,14 +62,14 @@ def test_a_set_beyond_the_chip_and_back(precision):
     """Requests of 20,160, 10,080 and 5,040 segments: alone or two small ones
     fit the chip (18,240), the three together and the largest do not, so ticks
     change between the two forms within one run, exchanges in both."""
-    reqs = [(I.channel(1000, 630), 0.7, 0.02, 1200, 0, 0),
-            (I.channel(1000, 315), 0.8, 0.02, 2000, 2, 40),
-            (np.ascontiguousarray(I.random_blobs(500, 317, 5, density=0.1)), 0.75, 0.02, 2600, 1, 30)]
+    reqs = [(I.channel(1000, 630), 0.7, 0.02, 6000, 0, 0),
+            (I.channel(1000, 315), 0.8, 0.02, 8000, 2, 40),
+            (np.ascontiguousarray(I.random_blobs(500, 317, 5, density=0.1)), 0.75, 0.02, 9000, 1, 30)]
     srv_calls = L.kernel_launches()
     done, stats = _serve(reqs, precision=precision, max_tick_steps=400)
     steps = sum(s * (1 + n) for _, _, _, s, n, _ in reqs)
     assert stats["peak_active"] == 3
     # between one launch a step (all per phase) and one a tick (all on the chip)
     launches = L.kernel_launches() - srv_calls
-    assert 1200 <= launches < steps
+    assert 6000 <= launches < steps
     _check_alone(reqs, done, precision)
